@@ -19,8 +19,12 @@
 // w, w^2, w^4, w^8 (compact; the other powers are products of at most three
 // of these, within a few units of rounding), w = exp(-2 pi i (j mod NS) /
 // (NS R)).
+//
+// Double precision runs the same stages in 64-bit fixed point (fft64.cuh);
+// its stage tables hold the twiddles as scaled integers.
 #pragma once
 #include "common.cuh"
+#include "fft64.cuh"
 
 namespace epfft {
 
@@ -302,13 +306,131 @@ __device__ __forceinline__ void fft_stages(C2<T>* s, const C2<T>* __restrict__ t
   }
 }
 
+// Largest of a value over the CTA's NT threads (every thread calls it; it
+// holds one barrier, and the caller another one before the next call).
+template <int NT>
+__device__ __forceinline__ unsigned block_max_u32(unsigned x) {
+  __shared__ unsigned wm[NT / 32];
+  x = __reduce_max_sync(0xffffffffu, x);
+  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = x;
+  __syncthreads();
+  unsigned m = wm[0];
+#pragma unroll
+  for (int i = 1; i < NT / 32; i++) m = max(m, wm[i]);
+  return m;
+}
+
+// The Stockham stage in fixed point (double sequences, fft64.cuh): the same
+// butterflies, addresses and barriers as stockham_stage.  The first stage
+// finds the block exponent of the NSEQ sequences and converts, the last one
+// rounds to doubles.  RENORM (N >= 1024): before every later stage the
+// integers are shifted up to the 62 bits again (the stages' divisions cost
+// sequences of few large numbers up to log2 N bits, which up to N = 512 still
+// leave an error below the FP64 butterflies').  emax: the block exponent.
+template <int N, int RM, bool FULL, int NSEQ, int NT, int K, bool INV>
+__device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>* __restrict__ tw, int& emax) {
+  using P = FftPlan<N, RM, FULL>;
+  constexpr int R = P::radix(K), NS = P::ns(K), LR = ilog2c(R);
+  constexpr int NJ = N / R, NBF = NSEQ * NJ, KB = (NBF + NT - 1) / NT, SP = seq_stride<N>();
+  constexpr bool FIRST = K == 0, LAST = K == P::NSTAGES - 1, RENORM = N >= 1024 && !FIRST;
+  C2<i64>* z = reinterpret_cast<C2<i64>*>(s);
+  C2<i64> v[KB][R];
+  const int tid = threadIdx.x;
+  unsigned mx = 0;
+#pragma unroll
+  for (int q = 0; q < KB; q++) {
+    const int g = tid + q * NT;
+    if (NBF % NT == 0 || g < NBF) {
+      const int j = g % NJ, sq = g / NJ;
+      const int rb = sq * SP + (NJ >= 32 ? pad32(j) : j);
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        v[q][r] = z[rb + read_off<N, R, NS>(r)];
+        const int hr = (int)(v[q][r].re >> 32), hi = (int)(v[q][r].im >> 32);
+        if constexpr (FIRST) mx = max(mx, max((unsigned)hr & 0x7fffffffu, (unsigned)hi & 0x7fffffffu));
+        if constexpr (RENORM) mx = max(mx, (unsigned)max(hr ^ (hr >> 31), hi ^ (hi >> 31)));
+      }
+    }
+  }
+  int sh = 0;
+  if constexpr (FIRST || RENORM) {
+    mx = block_max_u32<NT>(mx);
+    if constexpr (FIRST) {
+      emax = block_exp(mx);
+    } else {
+      sh = max(__clz((int)mx) - 2, 0);
+      if (emax >= 2047) sh = 0;
+      emax -= sh;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < KB; q++) {
+    const int g = tid + q * NT;
+    if (NBF % NT == 0 || g < NBF) {
+      const int j = g % NJ;
+      if constexpr (FIRST) {
+#pragma unroll
+        for (int r = 0; r < R; r++) {
+          v[q][r].re = to_fixed<LR>(__longlong_as_double(v[q][r].re), emax);
+          v[q][r].im = to_fixed<LR>(__longlong_as_double(v[q][r].im), emax);
+        }
+      } else {
+        if constexpr (RENORM) {
+#pragma unroll
+          for (int r = 0; r < R; r++) {
+            v[q][r].re = (i64)((unsigned long long)v[q][r].re << sh);
+            v[q][r].im = (i64)((unsigned long long)v[q][r].im << sh);
+          }
+        }
+        Tw64 w[R];
+        stage_twiddles64<R, NS, FULL>(reinterpret_cast<const Tw64*>(tw + P::tw_off(K)), j % NS, w);
+        v[q][0].re = rshift<LR>(v[q][0].re);
+        v[q][0].im = rshift<LR>(v[q][0].im);
+#pragma unroll
+        for (int r = 1; r < R; r++) cmul_hi<INV>(v[q][r].re, v[q][r].im, w[r]);
+      }
+      Bfly64<R, INV>::run(v[q]);
+    }
+  }
+  if constexpr (!(FIRST || RENORM)) __syncthreads();  // else block_max_u32's barrier followed every read
+#pragma unroll
+  for (int q = 0; q < KB; q++) {
+    const int g = tid + q * NT;
+    if (NBF % NT == 0 || g < NBF) {
+      const int j = g % NJ, sq = g / NJ;
+      const int jm = j % NS, a = (j / NS) * NS * R;
+      const int wb = sq * SP + (N < 32 ? a + jm : (NS <= 32 ? a + (a >> 5) + jm : pad32(a + jm)));
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const int i = wb + write_off<N, R, NS>(r);
+        if constexpr (LAST) s[i] = mk(from_fixed<ilog2c(N)>(v[q][r].re, emax), from_fixed<ilog2c(N)>(v[q][r].im, emax));
+        else z[i] = v[q][r];
+      }
+    }
+  }
+  __syncthreads();
+}
+
+template <int N, int RM, bool FULL, int NSEQ, int NT, bool INV, int K = 0>
+__device__ __forceinline__ void fft_stages64(C2<double>* s, const C2<double>* __restrict__ tw, int& emax) {
+  if constexpr (K < FftPlan<N, RM, FULL>::NSTAGES) {
+    stockham_stage64<N, RM, FULL, NSEQ, NT, K, INV>(s, tw, emax);
+    fft_stages64<N, RM, FULL, NSEQ, NT, INV, K + 1>(s, tw, emax);
+  }
+}
+
 // Transforms NSEQ sequences of length N (layout above) in place with the
 // plan FftPlan<N, RM, FULL> and its stage table tw (shared memory).  The
 // caller has completed the data and the table (barrier) before the call;
 // the call ends with a barrier.
 template <typename T, int N, int RM, bool FULL, int NSEQ, int NT, bool INV>
 __device__ __forceinline__ void fft_seq(C2<T>* s, const C2<T>* __restrict__ tw) {
-  fft_stages<T, N, RM, FULL, NSEQ, NT, INV>(s, tw);
+  if constexpr (sizeof(T) == 8) {
+    int emax = 0;
+    fft_stages64<N, RM, FULL, NSEQ, NT, INV>(s, tw, emax);
+  } else {
+    fft_stages<T, N, RM, FULL, NSEQ, NT, INV>(s, tw);
+  }
 }
 
 // Asynchronous global -> shared copy of one complex number (cp.async: the

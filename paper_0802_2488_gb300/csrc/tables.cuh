@@ -18,6 +18,8 @@
 //                         transform of length L/2 and its twists (RowPlan)
 // Variants with the same plans share their stage tables.
 #pragma once
+#include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "fft.cuh"
@@ -170,14 +172,35 @@ inline void host_expi(long n, long d, T* out) {
   out[1] = (T)(-sinl(a));
 }
 
-// Stage table of plan P at h (complex entries, interleaved reals).
+// exp(-2 pi i n / d) as balanced words of scale 2^S (Tw64 of fft64.cuh),
+// rounded once; the low word -2^31 is moved by one unit, so that the words
+// can change sign.
+inline Tw64 host_tw64(long n, long d, int S) {
+  const long double pi = 3.141592653589793238462643383279502884L;
+  const long double a = 2.0L * pi * (long double)(n % d) / (long double)d, sc = ldexpl(1.0L, S);
+  i64 re = llrintl(cosl(a) * sc), im = llrintl(-sinl(a) * sc);
+  if (bal_lo(re) == INT32_MIN) re += 1;
+  if (bal_lo(im) == INT32_MIN) im += 1;
+  return Tw64{bal_lo(re), bal_hi(re), bal_lo(im), bal_hi(im)};
+}
+
+// Stage table of plan P at h (complex entries: interleaved reals, or the
+// scaled integers of the fixed-point stages for double).
 template <typename T, typename P>
 inline void host_stage_table(T* h) {
   for (int k = 1; k < P::NSTAGES; k++) {
     const int R = P::radix(k), NS = P::ns(k);
     for (int p = 0; p < P::NP; p++) {
       const int pw = P::NP == R - 1 ? p + 1 : (1 << p);  // full: w^(p+1); compact: w^(2^p)
-      for (int jm = 0; jm < NS; jm++) host_expi<T>((long)jm * pw, (long)NS * R, h + 2 * (P::tw_off(k) + p * NS + jm));
+      for (int jm = 0; jm < NS; jm++) {
+        T* o = h + 2 * (P::tw_off(k) + p * NS + jm);
+        if constexpr (sizeof(T) == 8) {
+          const Tw64 w = host_tw64((long)jm * pw, (long)NS * R, 64 - ilog2c(R));
+          std::memcpy(o, &w, sizeof(w));
+        } else {
+          host_expi<T>((long)jm * pw, (long)NS * R, o);
+        }
+      }
     }
   }
 }
