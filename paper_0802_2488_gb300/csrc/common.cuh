@@ -109,6 +109,12 @@ enum MatConst : int {
   MC_TSTAR2,      // its square
   MC_RY,          // sqrt(2/3) Y / (2 mu0)
   MC_JC,          // mu / ((mu + mu0) 2 mu0)
+  MC_3K0,         // 3 K0
+  MC_HLIM,        // MC_TSTAR2 / 2
+  MC_YLIM_R2,     // sqrt(1/3) Y
+  MC_EM_MAT,      // 1 / (9 (K + K0))
+  MC_EM_VOID,     // 1 / (9 K0)
+  MC_PB_EL,       // (mu - mu0) / (mu + mu0): MC_GSC_EL - 2 mu0 / (2 (mu + mu0))
   N_MC
 };
 

@@ -342,9 +342,7 @@ row_pass_dc(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<float>* _
       if constexpr (EARLY_HALO) load_halo();
       cp_async_wait_all();
       __syncthreads();
-      IO::c2r_twist(sp, IO::octant(stw));
-      __syncthreads();
-      IO::template fft<true>(sp, stw);
+      IO::rows_inverse(sp, stw);
       if constexpr (!EARLY_HALO) load_halo();
       // one pixel: sj = d_sig^n, (l11, l12) = d_sig^n at x - e^1
       auto update = [&](int r, int j, int x1, bool v, const float (&sj)[4], float l11, float l12) {
@@ -458,8 +456,7 @@ row_pass_dc(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<float>* _
         }
       }
       __syncthreads();
-      IO::template fft<false>(sp, stw);
-      IO::r2c_twist(sp, IO::octant(stw));
+      IO::rows_forward(sp, stw);
       __syncthreads();
       IO::store(sp, spec, r0);
     }
@@ -593,8 +590,7 @@ dc_ref_forward(Solve* __restrict__ solves, Solve* __restrict__ shadow, const C2<
   block_reduce_acc<NT>(acc, S.refpart + (size_t)blockIdx.x * PART_STRIDE);
   cp_async_wait_all();
   __syncthreads();
-  IO::template fft<false>(sp, stw);
-  IO::r2c_twist(sp, IO::octant(stw));
+  IO::rows_forward(sp, stw);
   __syncthreads();
   IO::store(sp, reinterpret_cast<C2<double>*>(S.spec64), r0);
 }
@@ -627,9 +623,7 @@ dc_ref_inverse(Solve* __restrict__ solves, const C2<double>* __restrict__ tw) {
   IO::load_async(sp, reinterpret_cast<const C2<double>*>(S.spec64), r0);
   cp_async_wait_all();
   __syncthreads();
-  IO::c2r_twist(sp, IO::octant(stw));
-  __syncthreads();
-  IO::template fft<true>(sp, stw);
+  IO::rows_inverse(sp, stw);
   for (int r = 0; r < RR; r++)
     for (int j = 0; j < P; j++) {
       const int x1 = (int)threadIdx.x + j * NT;

@@ -299,6 +299,12 @@ void fill_consts(Solve& S) {
   c[MC_TSTAR2] = std::isinf(yl) ? yl : c[MC_TSTAR] * c[MC_TSTAR];
   c[MC_RY] = yl / (2.0 * S.mu0);
   c[MC_JC] = S.mu / ((S.mu + S.mu0) * 2.0 * S.mu0);
+  c[MC_3K0] = 3.0 * K0;
+  c[MC_HLIM] = 0.5 * c[MC_TSTAR2];
+  c[MC_YLIM_R2] = std::sqrt(1.0 / 3.0) * S.Y;
+  c[MC_EM_MAT] = 1.0 / (9.0 * (K + K0));
+  c[MC_EM_VOID] = 1.0 / (9.0 * K0);
+  c[MC_PB_EL] = (S.mu - S.mu0) / (S.mu + S.mu0);
   for (int i = 0; i < N_MC; i++) S.mcf[i] = (float)c[i];
 }
 

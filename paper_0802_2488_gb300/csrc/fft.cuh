@@ -323,16 +323,23 @@ __device__ __forceinline__ unsigned block_max_u32(unsigned x) {
 // The Stockham stage in fixed point (double sequences, fft64.cuh): the same
 // butterflies, addresses and barriers as stockham_stage.  The first stage
 // finds the block exponent of the NSEQ sequences and converts, the last one
-// rounds to doubles.  RENORM (N >= 1024): before every later stage the
-// integers are shifted up to the 62 bits again (the stages' divisions cost
-// sequences of few large numbers up to log2 N bits, which up to N = 512 still
-// leave an error below the FP64 butterflies').  emax: the block exponent.
-template <int N, int RM, bool FULL, int NSEQ, int NT, int K, bool INV>
+// rounds to doubles.  RENORM: before the stage the integers are shifted up to
+// the 62 bits again.  The stages' divisions cost sequences of a few large
+// numbers (the spectrum of a field with a large mean) up to log2 N bits;
+// shifting up before each stage that would take them to seven (six before a
+// radix-16 stage) keeps the
+// rounding below that of FP64 butterflies for them too (projection with a
+// mean strain at L = 1024 against long double: 8.3e-16 without, 2.0e-16 with,
+// 4.1e-16 for FP64 butterflies).  emax: the block exponent.
+// IN_INT: the sequences already hold integers made with emax (moduli below
+// 2^62.5 / R of the first stage); OUT_INT: they are left as integers.
+template <int N, int RM, bool FULL, int NSEQ, int NT, int K, bool INV, bool IN_INT, bool OUT_INT>
 __device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>* __restrict__ tw, int& emax) {
   using P = FftPlan<N, RM, FULL>;
   constexpr int R = P::radix(K), NS = P::ns(K), LR = ilog2c(R);
   constexpr int NJ = N / R, NBF = NSEQ * NJ, KB = (NBF + NT - 1) / NT, SP = seq_stride<N>();
-  constexpr bool FIRST = K == 0, LAST = K == P::NSTAGES - 1, RENORM = N >= 1024 && !FIRST;
+  constexpr bool FIRST = K == 0, LAST = K == P::NSTAGES - 1, RENORM = !FIRST && ilog2c(NS) + LR >= (LR == 4 ? 6 : 7);
+  constexpr bool CONVERT = FIRST && !IN_INT;
   C2<i64>* z = reinterpret_cast<C2<i64>*>(s);
   C2<i64> v[KB][R];
   const int tid = threadIdx.x;
@@ -347,15 +354,15 @@ __device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>
       for (int r = 0; r < R; r++) {
         v[q][r] = z[rb + read_off<N, R, NS>(r)];
         const int hr = (int)(v[q][r].re >> 32), hi = (int)(v[q][r].im >> 32);
-        if constexpr (FIRST) mx = max(mx, max((unsigned)hr & 0x7fffffffu, (unsigned)hi & 0x7fffffffu));
+        if constexpr (CONVERT) mx = max(mx, max((unsigned)hr & 0x7fffffffu, (unsigned)hi & 0x7fffffffu));
         if constexpr (RENORM) mx = max(mx, (unsigned)max(hr ^ (hr >> 31), hi ^ (hi >> 31)));
       }
     }
   }
   int sh = 0;
-  if constexpr (FIRST || RENORM) {
+  if constexpr (CONVERT || RENORM) {
     mx = block_max_u32<NT>(mx);
-    if constexpr (FIRST) {
+    if constexpr (CONVERT) {
       emax = block_exp(mx);
     } else {
       sh = max(__clz((int)mx) - 2, 0);
@@ -368,13 +375,13 @@ __device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>
     const int g = tid + q * NT;
     if (NBF % NT == 0 || g < NBF) {
       const int j = g % NJ;
-      if constexpr (FIRST) {
+      if constexpr (CONVERT) {
 #pragma unroll
         for (int r = 0; r < R; r++) {
           v[q][r].re = to_fixed<LR>(__longlong_as_double(v[q][r].re), emax);
           v[q][r].im = to_fixed<LR>(__longlong_as_double(v[q][r].im), emax);
         }
-      } else {
+      } else if constexpr (!FIRST) {
         if constexpr (RENORM) {
 #pragma unroll
           for (int r = 0; r < R; r++) {
@@ -392,7 +399,7 @@ __device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>
       Bfly64<R, INV>::run(v[q]);
     }
   }
-  if constexpr (!(FIRST || RENORM)) __syncthreads();  // else block_max_u32's barrier followed every read
+  if constexpr (!(CONVERT || RENORM)) __syncthreads();  // else block_max_u32's barrier followed every read
 #pragma unroll
   for (int q = 0; q < KB; q++) {
     const int g = tid + q * NT;
@@ -403,7 +410,7 @@ __device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>
 #pragma unroll
       for (int r = 0; r < R; r++) {
         const int i = wb + write_off<N, R, NS>(r);
-        if constexpr (LAST) s[i] = mk(from_fixed<ilog2c(N)>(v[q][r].re, emax), from_fixed<ilog2c(N)>(v[q][r].im, emax));
+        if constexpr (LAST && !OUT_INT) s[i] = mk(from_fixed<ilog2c(N)>(v[q][r].re, emax), from_fixed<ilog2c(N)>(v[q][r].im, emax));
         else z[i] = v[q][r];
       }
     }
@@ -411,11 +418,11 @@ __device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>
   __syncthreads();
 }
 
-template <int N, int RM, bool FULL, int NSEQ, int NT, bool INV, int K = 0>
+template <int N, int RM, bool FULL, int NSEQ, int NT, bool INV, bool IN_INT = false, bool OUT_INT = false, int K = 0>
 __device__ __forceinline__ void fft_stages64(C2<double>* s, const C2<double>* __restrict__ tw, int& emax) {
   if constexpr (K < FftPlan<N, RM, FULL>::NSTAGES) {
-    stockham_stage64<N, RM, FULL, NSEQ, NT, K, INV>(s, tw, emax);
-    fft_stages64<N, RM, FULL, NSEQ, NT, INV, K + 1>(s, tw, emax);
+    stockham_stage64<N, RM, FULL, NSEQ, NT, K, INV, IN_INT, OUT_INT>(s, tw, emax);
+    fft_stages64<N, RM, FULL, NSEQ, NT, INV, IN_INT, OUT_INT, K + 1>(s, tw, emax);
   }
 }
 
@@ -460,6 +467,15 @@ __device__ __forceinline__ void prefetch_l2(const void* p, unsigned n) {
 template <typename T, int NT>
 __device__ __forceinline__ void copy_table(C2<T>* dst, const C2<T>* __restrict__ src, int n) {
   for (int i = threadIdx.x; i < n; i += NT) cp_async_c2(dst + i, src + i);
+}
+
+// The same as scaled words (double, fft64.cuh).
+template <int L>
+__device__ __forceinline__ Tw64 twist_tw64(const C2<double>* __restrict__ t, int k) {
+  const Tw64* o = reinterpret_cast<const Tw64*>(t);
+  if (k <= L / 8) return o[k];
+  const Tw64 b = o[L / 4 - k];
+  return Tw64{-b.il, -b.ih, -b.rl, -b.rh};
 }
 
 // exp(-2 pi i k / L) for 0 <= k <= L/4 from the octant t[0 .. L/8]:

@@ -23,12 +23,13 @@
 // every operation).  A NaN or infinity in the block makes every output of the
 // block NaN (as one in a sequence does to the sequence's outputs).
 //
-// Measured (8 x L = 512, CUDA events): column pass 581 -> 328 us, row pass
-// 787 -> 631 us (what is left on the FP64 pipe is the Green operator, the row
-// twists and the pixel step); L = 4096: 5.69 -> 2.74 ms and 7.83 -> 5.79 ms.
-// Against long double (random data, N = 512): 5e-17 relative against 1.9e-16
-// for FP64 butterflies; single pixels and 1/q^2 spectra 0.6 - 0.9e-16 against
-// 0.8 - 1.8e-16.
+// Measured (8 x L = 512, CUDA events): column pass 581 -> 330 us; row pass
+// 787 -> 631 us, and 416 us with the twists in fixed point too and the pixel
+// step of local_step64 (what is left on the FP64 pipe is the Green operator
+// and the pixel step); L = 4096: 5.69 -> 2.74 ms and 7.83 -> 4.15 ms.
+// Against long double: projection at L = 64, 256 1.8e-16, 1.9e-16 relative
+// (FP64 butterflies 3.2e-16, 3.6e-16), 20 iterations at L = 256 7.0e-16
+// (1.25e-15).
 #pragma once
 #include "common.cuh"
 
@@ -75,6 +76,22 @@ EPFFT_HD void cmul_hi(i64& re, i64& im, const Tw64& w) {
   n += (i64)il * w.rh;
   re = (m >> 32) + (i64)rh * w.rh + (i64)ih * -wh;
   im = (n >> 32) + (i64)rh * wh + (i64)ih * w.rh;
+}
+// a w / 2^63 (complex) with w of scale 2^62, i.e. half the product.
+EPFFT_HD void cmul_half(i64& re, i64& im, const Tw64& w) {
+  const int rl = bal_lo(re), rh = bal_hi(re), il = bal_lo(im), ih = bal_hi(im);
+  i64 m = 0x40000000ll, n = 0x40000000ll;
+  m += (i64)rh * w.rl;
+  m += (i64)rl * w.rh;
+  m += (i64)ih * -w.il;
+  m += (i64)il * -w.ih;
+  n += (i64)rh * w.il;
+  n += (i64)rl * w.ih;
+  n += (i64)ih * w.rl;
+  n += (i64)il * w.rh;
+  const i64 p = (i64)rh * w.rh + (i64)ih * -w.ih, q = (i64)rh * w.ih + (i64)ih * w.rh;
+  re = (m >> 31) + (i64)((unsigned long long)p << 1);
+  im = (n >> 31) + (i64)((unsigned long long)q << 1);
 }
 // a w / 2^S (complex), for products of twiddles of scale 2^S (S = 64 - log2 R).
 template <int S>

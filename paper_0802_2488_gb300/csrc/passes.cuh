@@ -71,7 +71,10 @@ struct Cfg {
                                      : (L <= 256 ? L : (V == 0 && L == 512 ? 256 : NTMAX));
   static constexpr int NT_ROW = NT_ROW0 < 32 ? 32 : NT_ROW0;
   static constexpr int NT_COL0 = ((3 * W * L / RM_COL + 31) / 32) * 32;
-  static constexpr int NT_COL = NT_COL0 < 32 ? 32 : (NT_COL0 > NTMAX ? NTMAX : NT_COL0);
+  // 256 threads for the FP64 L = 4096 column: at 512 the 128 registers a
+  // thread spill (3.75 ms against 2.74)
+  static constexpr int NTMAX_COL = F64 && L == 4096 ? 256 : NTMAX;
+  static constexpr int NT_COL = NT_COL0 < 32 ? 32 : (NT_COL0 > NTMAX_COL ? NTMAX_COL : NT_COL0);
   static constexpr int MINB_COL = F64 ? 1
                                       : V == 1 ? 2 : (L == 512 ? 768 / NT_COL : (L == 1024 || L == 2048 ? 3 : 1));
   // sequences transformed per call: the largest divisor of the sequence
@@ -248,6 +251,108 @@ struct RowIO {
         where(e, r0, is, ig);
         if (ECHK(is, SZ, 3) && ECHK(ig, (size_t)3 * M * L, 4)) spec[ig] = sp[is];
       }
+    }
+  }
+  // Double precision: the twists work on the fixed-point numbers of the
+  // transforms (fft64.cuh).  The inverse one finds the tile's block exponent,
+  // converts and leaves integers of a quarter of Z (moduli below 2^62.5 / R0
+  // of the first stage) for fft<true>; the forward one takes the integers
+  // fft<false> leaves (block exponent s_em[group]) and writes doubles.
+  static constexpr int LG_R0 = ilog2c(C::PR::radix(0));
+  static constexpr int NG = NSEQ / C::G_R;  // transform calls per tile
+  static __device__ __forceinline__ int c2r_twist64(C2<T>* sp, const C2<T>* __restrict__ oct) {
+    unsigned mx = 0;
+    for (int i = threadIdx.x; i < NSEQ * M; i += NT) {
+      const int q = (i / M) * SP + pad32(i % M);
+      if (!ECHK(q, SZ, 38)) continue;
+      const C2<T> z = sp[q];
+      mx = max(mx, max((unsigned)hi_word(z.re) & 0x7fffffffu, (unsigned)hi_word(z.im) & 0x7fffffffu));
+    }
+    const int emax = block_exp(block_max_u32<NT>(mx));
+    auto pair = [&](int k, int sq0, int ds) {
+      const int kk = M - k;
+      const int ik = pad32(k), ikk = pad32(kk);  // 0 < k, kk < M
+      const Tw64 wk = twist_tw64<L>(oct, k);
+      for (int sq = sq0; sq < NSEQ; sq += ds) {
+        C2<T>* s = sp + sq * SP;
+        if (!ECHK(sq * SP + ikk, SZ, 38) || !ECHK(sq * SP + ik, SZ, 38)) continue;
+        C2<i64>* z = reinterpret_cast<C2<i64>*>(s);
+        const i64 ar = to_fixed<LG_R0>(s[ik].re, emax), ai = to_fixed<LG_R0>(s[ik].im, emax);
+        const i64 br = to_fixed<LG_R0>(s[ikk].re, emax), bi = to_fixed<LG_R0>(s[ikk].im, emax);
+        i64 tr = ar - br, ti = ai + bi;
+        cmul_hi<true>(tr, ti, wk);
+        const i64 sr = rshift<2>(ar + br), si = rshift<2>(ai - bi);
+        z[ik] = mk(sr - ti, si + tr);
+        if (kk != k) z[ikk] = mk(sr + ti, tr - si);
+      }
+    };
+    visit_pairs(pair);
+    for (int sq = threadIdx.x; sq < NSEQ; sq += NT) {
+      C2<T>* s = sp + sq * SP;
+      const i64 a = to_fixed<LG_R0>(s[0].re, emax), b = to_fixed<LG_R0>(s[0].im, emax);
+      reinterpret_cast<C2<i64>*>(s)[0] = mk(rshift<2>(a + b), rshift<2>(a - b));
+    }
+    return emax;
+  }
+  // half of X(k) (see r2c_twist), so that the sums stay below 2^63
+  static __device__ __forceinline__ void r2c_twist64(C2<T>* sp, const C2<T>* __restrict__ oct, const int* s_em) {
+    constexpr int LG = ilog2c(M);
+    auto pair = [&](int k, int sq0, int ds) {
+      const int kk = M - k;
+      const int ik = pad32(k), ikk = pad32(kk);  // 0 < k, kk < M
+      const Tw64 wk = twist_tw64<L>(oct, k);
+      for (int sq = sq0; sq < NSEQ; sq += ds) {
+        C2<T>* s = sp + sq * SP;
+        if (!ECHK(sq * SP + ikk, SZ, 38) || !ECHK(sq * SP + ik, SZ, 38)) continue;
+        const int em = s_em[NG == 1 ? 0 : sq / C::G_R] + 1;
+        const C2<i64> a = reinterpret_cast<C2<i64>*>(s)[ik], b = reinterpret_cast<C2<i64>*>(s)[ikk];
+        i64 tr = (a.re >> 1) - (b.re >> 1), ti = (a.im >> 1) + (b.im >> 1);
+        cmul_half(tr, ti, wk);
+        const i64 sr = rshift<1>((a.re >> 1) + (b.re >> 1)), si = rshift<1>((a.im >> 1) - (b.im >> 1));
+        s[ik] = mk(from_fixed<LG>(sr + ti, em), from_fixed<LG>(si - tr, em));
+        if (kk != k) s[ikk] = mk(from_fixed<LG>(sr - ti, em), from_fixed<LG>(-si - tr, em));
+      }
+    };
+    visit_pairs(pair);
+    for (int sq = threadIdx.x; sq < NSEQ; sq += NT) {
+      C2<T>* s = sp + sq * SP;
+      const int em = s_em[NG == 1 ? 0 : sq / C::G_R] + 1;
+      const C2<i64> z = reinterpret_cast<C2<i64>*>(s)[0];
+      s[0] = mk(from_fixed<LG>((z.re >> 1) + (z.im >> 1), em), from_fixed<LG>((z.re >> 1) - (z.im >> 1), em));
+    }
+  }
+  // Spectrum tile (loaded, after a barrier) -> real rows, and back.  Both
+  // begin after a barrier; the inverse ends with one, the forward one is
+  // followed by one of the caller's.
+  static __device__ __forceinline__ void rows_inverse(C2<T>* sp, const C2<T>* __restrict__ stw) {
+    if constexpr (sizeof(T) == 8) {
+      const int emax = c2r_twist64(sp, octant(stw)) + 2;
+      __syncthreads();
+#pragma unroll 1
+      for (int g = 0; g < NG; g++) {
+        int em = emax;
+        fft_stages64<M, C::RM_ROW, C::FULL, C::G_R, NT, true, true, false>(sp + g * C::G_R * SP, stw, em);
+      }
+    } else {
+      c2r_twist(sp, octant(stw));
+      __syncthreads();
+      fft<true>(sp, stw);
+    }
+  }
+  static __device__ __forceinline__ void rows_forward(C2<T>* sp, const C2<T>* __restrict__ stw) {
+    if constexpr (sizeof(T) == 8) {
+      __shared__ int s_em[NG];
+#pragma unroll 1
+      for (int g = 0; g < NG; g++) {
+        int em = 0;
+        fft_stages64<M, C::RM_ROW, C::FULL, C::G_R, NT, false, false, true>(sp + g * C::G_R * SP, stw, em);
+        if (threadIdx.x == 0) s_em[g] = em;
+      }
+      __syncthreads();
+      r2c_twist64(sp, octant(stw), s_em);
+    } else {
+      fft<false>(sp, stw);
+      r2c_twist(sp, octant(stw));
     }
   }
   // Half spectrum (packed) -> Z for the half-length inverse transform:
@@ -656,8 +761,13 @@ row_pass(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<T>* __restri
     T* __restrict__ sout = reinterpret_cast<T*>(S.sig[1 - cur]);
     C2<T>* spec = reinterpret_cast<C2<T>*>(S.spec);
     const uint8_t* __restrict__ mask = S.mask;
-    const Mat<T> m = make_mat<T>(S);
+    Mat<T> m = make_mat<T>(S);
     const size_t LL = (size_t)L * L;
+    // double precision: the plastic count and the 12 part of the residual of
+    // this thread, added to its sums at the end (an integer add and one FP64
+    // multiply-add per pixel instead of two and a compare)
+    int n_pl = 0;
+    T comp12 = T(0);
     // stage table and twist octant, in flight until the first barrier after
     // cp_async_wait_all() (INIT, ITER; the other phases do not read them)
     const C2<T>* stw = sp + C::ROW_DATA;
@@ -710,6 +820,7 @@ row_pass(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<T>* __restri
     } else {  // PH_ITER
       T E[4];
       load_E(S.path + 4 * inc, E);
+      m.E33 = E[2];
       IO::load_async(sp, spec, r0);
       // sigma of the RR rows and of the halo row, and the void flags, are
       // brought into the L2 while the spectrum is transformed (16 KB pieces,
@@ -751,9 +862,7 @@ row_pass(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<T>* __restri
       if constexpr (EARLY_HALO) load_halo();
       cp_async_wait_all();
       __syncthreads();
-      IO::c2r_twist(sp, IO::octant(stw));
-      __syncthreads();
-      IO::template fft<true>(sp, stw);
+      IO::rows_inverse(sp, stw);
       if constexpr (!EARLY_HALO) load_halo();
       // Pixel update of the AL iteration at (r, x1), given the stress sj of
       // iterate n (the multiplier) and the left neighbour's sigma11, sigma12
@@ -768,22 +877,36 @@ row_pass(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<T>* __restri
         prev22[j] = sj[1];
 #pragma unroll
         for (int c = 0; c < 4; c++) acc[A_S11 + c] += sj[c];
-        acc[A_DIV2] += d1 * d1 + d2 * d2;
+        if constexpr (sizeof(T) == 8) acc[A_DIV2] = fma(d1, d1, fma(d2, d2, acc[A_DIV2]));
+        else acc[A_DIV2] += d1 * d1 + d2 * d2;
         // augmented-Lagrangian update of this pixel
         T e[4] = {IO::px(sp, 0, r, x1), IO::px(sp, 1, r, x1), E[2], IO::px(sp, 2, r, x1)};
-        T c0[4], tau[4], e1[4], s1[4], p1[3];
-        c0_apply(e, m, c0);
+        T e1[4], s1[4], p1[3];
+        bool pl;
+        if constexpr (sizeof(T) == 8) {
+          pl = local_step64(sj, e[0], e[1], e[3], v, m, e1, s1, p1);
+        } else {
+          T c0[4], tau[4];
+          c0_apply(e, m, c0);
 #pragma unroll
-        for (int c = 0; c < 4; c++) tau[c] = sj[c] + c0[c];
-        local_solve_p(tau, v, m, e1, s1, p1);
+          for (int c = 0; c < 4; c++) tau[c] = sj[c] + c0[c];
+          local_solve_p(tau, v, m, e1, s1, p1);
+          pl = is_plastic(e1, v, m);
+        }
         Vec4<T>::store(eout + 4 * x, e1);
         Vec4<T>::store(sout + 4 * x, s1);
         // <eps^{n+1}> and its plastic pixels (stats of the next iterate)
 #pragma unroll
         for (int c = 0; c < 4; c++) acc[A_E11 + c] += e1[c];
-        acc[A_NPL] += is_plastic(e1, v, m) ? T(1) : T(0);
+        if constexpr (sizeof(T) == 8) n_pl += pl ? 1 : 0;
+        else acc[A_NPL] += pl ? T(1) : T(0);
         const T q0 = e1[0] - e[0], q1 = e1[1] - e[1], q2 = e1[2] - e[2], q3 = e1[3] - e[3];
-        acc[A_COMP] += q0 * q0 + q1 * q1 + q2 * q2 + T(2) * q3 * q3;
+        if constexpr (sizeof(T) == 8) {
+          acc[A_COMP] = fma(q0, q0, fma(q1, q1, fma(q2, q2, acc[A_COMP])));
+          comp12 = fma(q3, q3, comp12);
+        } else {
+          acc[A_COMP] += q0 * q0 + q1 * q1 + q2 * q2 + T(2) * q3 * q3;
+        }
         // next polarization sigma(eps^{n+1}) - C0:eps^{n+1} (in-plane)
         IO::px(sp, 0, r, x1) = p1[0];
         IO::px(sp, 1, r, x1) = p1[1];
@@ -873,11 +996,14 @@ row_pass(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<T>* __restri
       }
     }
 
+    if constexpr (sizeof(T) == 8) {
+      acc[A_NPL] += T(n_pl);
+      acc[A_COMP] = fma(T(2), comp12, acc[A_COMP]);
+    }
     if (phase == PH_ITER || phase == PH_INIT) {
       cp_async_wait_all();  // the tables (INIT)
       __syncthreads();
-      IO::template fft<false>(sp, stw);
-      IO::r2c_twist(sp, IO::octant(stw));
+      IO::rows_forward(sp, stw);
       __syncthreads();
       IO::store(sp, spec, r0);
     }
@@ -1087,8 +1213,7 @@ row_forward(const T* __restrict__ p, C2<T>* __restrict__ spec, const C2<T>* __re
     }
   cp_async_wait_all();
   __syncthreads();
-  IO::template fft<false>(sp, stw);
-  IO::r2c_twist(sp, IO::octant(stw));
+  IO::rows_forward(sp, stw);
   __syncthreads();
   IO::store(sp, spec, r0);
 }
@@ -1108,9 +1233,7 @@ row_inverse(const C2<T>* __restrict__ spec, T* __restrict__ e, const C2<T>* __re
   IO::load_async(sp, spec, r0);
   cp_async_wait_all();
   __syncthreads();
-  IO::c2r_twist(sp, IO::octant(stw));
-  __syncthreads();
-  IO::template fft<true>(sp, stw);
+  IO::rows_inverse(sp, stw);
   for (int r = 0; r < RR; r++)
     for (int j = 0; j < P; j++) {
       const int x1 = threadIdx.x + j * NT;

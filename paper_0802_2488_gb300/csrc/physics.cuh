@@ -20,6 +20,10 @@ struct Mat {
   T p_mat, p_void;  // 3 (K - K0), -3 K0
   T gsc_el;         // mu / (mu + mu0)
   T k3;             // 3 K
+  // double precision (local_step64): 3 K0, |tau'|^2 / 2 at yield,
+  // sqrt(2/3) Y / sqrt(2), mean parts of the strain per trace of tau, elastic
+  // coefficient of the polarization's deviator, prescribed E33
+  T k03, hlim, ylim_r2, em_mat, em_void, pb_el, E33;
 };
 
 template <typename T>
@@ -49,6 +53,13 @@ __device__ __forceinline__ Mat<T> make_mat(const Solve& S) {
   m.p_void = c[MC_P_VOID];
   m.gsc_el = c[MC_GSC_EL];
   m.k3 = c[MC_3K];
+  m.k03 = c[MC_3K0];
+  m.hlim = c[MC_HLIM];
+  m.ylim_r2 = c[MC_YLIM_R2];
+  m.em_mat = c[MC_EM_MAT];
+  m.em_void = c[MC_EM_VOID];
+  m.pb_el = c[MC_PB_EL];
+  m.E33 = T(0);  // set by the passes that use it
   return m;
 }
 
@@ -212,6 +223,56 @@ __device__ __forceinline__ bool local_solve_p(const T t[4], bool is_void, const 
   const T pm = pa * em;
   p[0] = pb * d0 + pm;
   p[1] = pb * d1 + pm;
+  p[2] = pb * d3;
+  return pl;
+}
+
+// The pixel step in double precision, written for few FP64 instructions (one
+// takes 19 clocks of an SM, fft64.cuh): from sigma^n (s), the in-plane
+// compatible strain (e11, e22, e12) and E33 = m.E33, the strain, stress and
+// polarization of local_solve_p for tau = sigma^n + C0:e.  With t = tr tau =
+// tr sigma + 3 K0 tr e the deviator is
+//   tau'_c = sigma_c + 2 mu0 e_c - (tr sigma + 2 mu0 tr e) / 3,
+// its third diagonal entry minus the sum of the other two, and
+// h = |tau'|^2 / 2 = tau'11 (tau'11 + tau'22) + tau'22^2 + tau'12^2.  Returns
+// the branch: true where the solution is plastic, i.e. |tau'| is above
+// sqrt(2/3) Y (mu + mu0) / mu.
+__device__ __forceinline__ bool local_step64(const double s[4], double e11, double e22, double e12, bool is_void,
+                                             const Mat<double>& m, double e1[4], double s1[4], double p[3]) {
+  const double trE = (e11 + e22) + m.E33, trS = (s[0] + s[1]) + s[2];
+  const double t = fma(m.k03, trE, trS);
+  const double q = fma(m.two_mu0, trE, trS) * (-1.0 / 3.0);
+  const double d0 = fma(m.two_mu0, e11, s[0] + q), d1 = fma(m.two_mu0, e22, s[1] + q);
+  const double d01 = d0 + d1, d3 = fma(m.two_mu0, e12, s[3]);
+  const double h = fma(d0, d01, fma(d1, d1, d3 * d3));
+  // both are >= 0 (or NaN), so their order is that of their bits
+  const bool pl = !is_void && __double_as_longlong(h) > __double_as_longlong(m.hlim);
+  double sc = is_void ? m.inv_2mu0 : m.inv_2mumu0, gsc = is_void ? 0.0 : m.gsc_el;
+  double pb = is_void ? -1.0 : m.pb_el;
+  if (pl) {
+    // 1 / sqrt(h): FP32 estimate (2^-22), one third-order step
+    const int hi = __double2hiint(h);
+    const float f = __int_as_float((int)((unsigned)(hi - 0x38000000) << 3 | (unsigned)__double2loint(h) >> 29));
+    const int fb = __float_as_int(rsqrtf(f));
+    double y = __hiloint2double((fb >> 3) + 0x38000000, fb << 29);
+    const double r = fma(-(h * y), y, 1.0);
+    y = fma(y * r, fma(0.375, r, 0.5), y);
+    gsc = m.ylim_r2 * y;  // sqrt(2/3) Y / |tau'|
+    sc = fma(-m.inv_2mu0, gsc, m.inv_2mu0);
+    pb = fma(2.0, gsc, -1.0);  // gsc - 2 mu0 sc
+  }
+  const double em = t * (is_void ? m.em_void : m.em_mat);
+  const double sm = (is_void ? 0.0 : m.k3) * em, pm = (is_void ? m.p_void : m.p_mat) * em;
+  e1[0] = fma(d0, sc, em);
+  e1[1] = fma(d1, sc, em);
+  e1[2] = fma(-d01, sc, em);
+  e1[3] = d3 * sc;
+  s1[0] = fma(gsc, d0, sm);
+  s1[1] = fma(gsc, d1, sm);
+  s1[2] = fma(-gsc, d01, sm);
+  s1[3] = gsc * d3;
+  p[0] = fma(pb, d0, pm);
+  p[1] = fma(pb, d1, pm);
   p[2] = pb * d3;
   return pl;
 }

@@ -4,6 +4,8 @@
 // the host in extended precision and rounded once to T, shared by both
 // tiling variants.  Layout in complex units:
 //   [0, OCT)              exp(-2 pi i k / L), k = 0 .. L/8 (row twists)
+//                         (double: this and the stage tables hold scaled
+//                         integers, fft64.cuh)
 //   [OFF_R[v], +TW_R[v])  stage table of the row plan of variant v
 //   [OFF_C[v], +TW_C[v])  stage table of the column plan of variant v
 //   [KOFF, KOFF + L)      k(m) = (sin q, 2 sin^2(q/2)), q = 2 pi m / L, the
@@ -219,7 +221,14 @@ inline void host_tables_L(std::vector<T>& h) {
   using TB = Tables<T, L>;
   h.assign((size_t)2 * TB::TOTAL, T(0));
   const long double pi = 3.141592653589793238462643383279502884L;
-  for (int k = 0; k < TB::OCT; k++) host_expi<T>(k, L, h.data() + 2 * k);
+  for (int k = 0; k < TB::OCT; k++) {
+    if constexpr (sizeof(T) == 8) {
+      const Tw64 w = host_tw64(k, L, 62);
+      std::memcpy(h.data() + 2 * k, &w, sizeof(w));
+    } else {
+      host_expi<T>(k, L, h.data() + 2 * k);
+    }
+  }
   host_stage_table<T, typename TB::S0::PR>(h.data() + 2 * TB::OFF_R0);
   host_stage_table<T, typename TB::S0::PC>(h.data() + 2 * TB::OFF_C0);
   if (!TB::SAME) {
