@@ -26,6 +26,9 @@ namespace {
 struct Server;
 }
 
+// instantiation units that hold a self-check record
+constexpr int N_CHECK_UNITS = 10;
+
 struct epfft_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;  // work stream
@@ -35,7 +38,7 @@ struct epfft_ctx {
   // page-locked copies of the self-check records of the instantiation units
   // and the records' device addresses (serving reads them on its stream)
   CheckRec* h_checks = nullptr;
-  void* check_addr[8] = {};
+  void* check_addr[N_CHECK_UNITS] = {};
   bool own_stream = false;
   epfft_alloc_fn alloc = nullptr;
   epfft_free_fn freef = nullptr;
@@ -52,6 +55,8 @@ struct epfft_ctx {
   // tuned tiling per (L, precision, batch class): class 1 when a launch
   // covers at least 2^21 pixels (enough CTAs to fill the GPU), else 0
   std::map<std::tuple<int, int, int>, int> variant;
+  // resident schedule: CTAs the GPU holds at once per (L, precision, tiling)
+  std::map<std::tuple<int, int, int>, int> res_cap;
   epfft_stats last{};
   Server* server = nullptr;
   // defect-correction form: iterations of a solve between refreshes of its
@@ -164,7 +169,7 @@ int get_tables(epfft_ctx* c, int L, int prec, void** tw, void** ktab) {
 
 // First recorded self-check failure of any instantiation unit.
 cudaError_t read_check_all(CheckRec* out) {
-  CheckRec r[8];
+  CheckRec r[N_CHECK_UNITS];
   cudaError_t e;
   if ((e = read_check_v<float, 0>(&r[0])) != cudaSuccess) return e;
   if ((e = read_check_v<float, 1>(&r[1])) != cudaSuccess) return e;
@@ -174,6 +179,8 @@ cudaError_t read_check_all(CheckRec* out) {
   if ((e = read_check_def_v<0>(&r[5])) != cudaSuccess) return e;
   if ((e = read_check_def_v<1>(&r[6])) != cudaSuccess) return e;
   if ((e = read_check_onchip(&r[7])) != cudaSuccess) return e;
+  if ((e = read_check_resident<float>(&r[8])) != cudaSuccess) return e;
+  if ((e = read_check_resident<double>(&r[9])) != cudaSuccess) return e;
   *out = CheckRec{};
   for (auto& x : r)
     if (x.code) {
@@ -189,7 +196,7 @@ cudaError_t read_check_all(CheckRec* out) {
 cudaError_t enqueue_check_reads(epfft_ctx* c, cudaStream_t s) {
   if (!c->h_checks) {
     cudaError_t e;
-    void* a[8] = {};
+    void* a[N_CHECK_UNITS] = {};
     if ((e = check_record_v<float, 0>(&a[0])) != cudaSuccess) return e;
     if ((e = check_record_v<float, 1>(&a[1])) != cudaSuccess) return e;
     if ((e = check_record_v<double, 0>(&a[2])) != cudaSuccess) return e;
@@ -198,15 +205,17 @@ cudaError_t enqueue_check_reads(epfft_ctx* c, cudaStream_t s) {
     if ((e = check_record_def_v<0>(&a[5])) != cudaSuccess) return e;
     if ((e = check_record_def_v<1>(&a[6])) != cudaSuccess) return e;
     if ((e = check_record_onchip(&a[7])) != cudaSuccess) return e;
+    if ((e = check_record_resident<float>(&a[8])) != cudaSuccess) return e;
+    if ((e = check_record_resident<double>(&a[9])) != cudaSuccess) return e;
     CheckRec* h = nullptr;
-    if ((e = cudaMallocHost((void**)&h, sizeof(CheckRec) * 8)) != cudaSuccess) return e;
-    for (int i = 0; i < 8; i++) {
+    if ((e = cudaMallocHost((void**)&h, sizeof(CheckRec) * N_CHECK_UNITS)) != cudaSuccess) return e;
+    for (int i = 0; i < N_CHECK_UNITS; i++) {
       c->check_addr[i] = a[i];
       h[i] = CheckRec{};
     }
     c->h_checks = h;
   }
-  for (int i = 0; i < 8; i++) {
+  for (int i = 0; i < N_CHECK_UNITS; i++) {
     if (!c->check_addr[i]) continue;
     cudaError_t e = cudaMemcpyAsync(&c->h_checks[i], c->check_addr[i], sizeof(CheckRec), cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return e;
@@ -325,6 +334,7 @@ struct Batch {
   int var64 = 0;
   Solve* d_shadow = nullptr;
   std::vector<Solve> h_shadow;  // serving: host copy of the shadow slots
+  bool resident = false;  // ran on the resident schedule
   int64_t refreshes = 0;  // refreshes launched from the host (fixed-step loops)
   std::vector<Solve> h_solves;
   std::vector<int32_t> n_inc;
@@ -631,6 +641,52 @@ int build_loop_graph(epfft_ctx* c, Batch& B, cudaGraph_t* graph_out, cudaGraphEx
   }
   *graph_out = graph;
   *exec_out = exec;
+  return EPFFT_OK;
+}
+
+// CTAs per solve of the resident schedule for a batch (resident.cuh), 0 where
+// the two-pass loop runs instead.  Sizes: those resident_supported names.
+// Batches: up to twice as many rows units as the GPU holds CTAs, i.e. at most
+// two or so per CTA; beyond, the passes' launches are amortised and their CTAs
+// overlap better (FP32 L = 64: 32 lattices 15 against 22 us an iteration, one
+// 9.8 against 20; L = 512: one 25 against 31, four 65 against 67).
+int resident_ctas(epfft_ctx* c, int L, int prec, int var, int nb, int row_ctas) {
+  if (prec == EPFFT_FP32 ? !resident_supported<float>(L, var)
+                         : prec != EPFFT_FP64 || !resident_supported<double>(L, var))
+    return 0;
+  const auto key = std::make_tuple(L, prec, var);
+  auto it = c->res_cap.find(key);
+  if (it == c->res_cap.end()) {
+    int per_sm = 0, nsm = 0, coop = 0;
+    const cudaError_t e = prec == EPFFT_FP32 ? prepare_resident<float>(L, var, &per_sm)
+                                             : prepare_resident<double>(L, var, &per_sm);
+    if (e != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device) != cudaSuccess || !coop) {
+      cudaGetLastError();
+      per_sm = 0;
+    }
+    it = c->res_cap.emplace(key, per_sm * nsm).first;
+  }
+  const int64_t cap = it->second;
+  if (cap < 1 || (int64_t)nb * row_ctas > 2 * cap) return 0;
+  int g = 1;
+  while (2 * g <= row_ctas && (int64_t)2 * g * nb <= cap) g *= 2;
+  return (int64_t)g * nb <= cap ? g : 0;
+}
+
+// Enqueues the resident schedule of a batch (g CTAs per solve).
+int enqueue_resident(epfft_ctx* c, Arena& A, Batch& B, int g) {
+  const size_t part = sizeof(double) * PART_STRIDE * (size_t)B.sh.row_ctas * (size_t)B.nb;
+  const size_t bar = 128 * (size_t)B.nb;
+  double* part2 = (double*)A.get(part);
+  unsigned* bars = (unsigned*)A.get(bar);
+  if (!part2 || !bars) return EPFFT_ERR_OOM;
+  CK(cudaMemsetAsync(bars, 0, bar, c->stream));
+  if (B.prec == EPFFT_FP64)
+    CK(launch_resident<double>(B.L, B.var, g, B.nb, c->stream, B.d_solves, B.d_ctl, part2, bars, B.tw, B.ktab, B.general));
+  else
+    CK(launch_resident<float>(B.L, B.var, g, B.nb, c->stream, B.d_solves, B.d_ctl, part2, bars, B.tw, B.ktab, B.general));
+  B.resident = true;
   return EPFFT_OK;
 }
 
@@ -984,6 +1040,9 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
   int rc = EPFFT_OK;
   if (chk && chk[0] == '1') {
     for (int g = 0; g < G && !rc; g++) rc = run_checked(c, Bs[g]);
+  } else if (const int g = G == 1 ? resident_ctas(c, Bs[0].L, Bs[0].prec, Bs[0].var, Bs[0].nb, Bs[0].sh.row_ctas) : 0) {
+    rc = enqueue_resident(c, A, Bs[0], g);
+    if (!rc && cudaStreamSynchronize(c->stream) != cudaSuccess) rc = EPFFT_ERR_CUDA;
   } else if (host_steps > 0) {
     rc = run_host_loop(c, Bs[0], host_steps);
   } else {
@@ -1052,8 +1111,9 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
       }
       streaming++;
       steps = std::max<int64_t>(steps, bc[g].body_iters);
-      // per step a column and a row pass of every batch
-      k += 2 * bc[g].body_iters;
+      // per step a column and a row pass of every batch; the resident
+      // schedule is one launch
+      k += Bs[g].resident ? 1 : 2 * bc[g].body_iters;
     }
     if (streaming > 1) k += steps;  // the loop-condition kernel of the mixed graph
     // the defect form's refreshes: from the host, and the loop body's node
@@ -1196,6 +1256,40 @@ int time_passes_impl(epfft_ctx* ctx, epfft_problem p, int n_batch, const double 
   *col_ms = (float)(tc / n_iter);
   *row_ms = (float)(tr / n_iter);
   return EPFFT_OK;
+}
+
+// Time per iteration (ms) of a solve of n_batch copies of p on the resident
+// schedule with tiling var: one launch of n_iter iterations.  *ms = 0 where
+// that batch runs the two-pass loop.
+int time_resident(epfft_ctx* ctx, epfft_problem p, int n_batch, const double E[4], int n_iter, int var, float* ms) {
+  *ms = 0.f;
+  if (cudaSetDevice(ctx->device) != cudaSuccess) return EPFFT_ERR_CUDA;
+  PassShape sh;
+  if (var == ONCHIP_VARIANT || shape(p.L, p.precision, var, &sh) != EPFFT_OK) return EPFFT_OK;
+  const int g = resident_ctas(ctx, p.L, p.precision, var, n_batch, sh.row_ctas);
+  if (!g) return EPFFT_OK;
+  p.tol_eq = p.tol_macro = 0.0;
+  p.max_iter = n_iter;
+  std::vector<epfft_problem> ps(n_batch, p);
+  std::vector<epfft_path> paths(n_batch, epfft_path{1, 0, E});
+  Arena A(ctx);
+  Batch B;
+  B.var = var;
+  int rc = setup_batch(ctx, A, B, n_batch, ps.data(), paths.data(), nullptr);
+  if (rc) return rc;
+  cudaEvent_t e0, e1;
+  CK(cudaEventCreate(&e0));
+  CK(cudaEventCreate(&e1));
+  CK(cudaEventRecord(e0, ctx->stream));
+  rc = enqueue_resident(ctx, A, B, g);
+  if (!rc && (cudaEventRecord(e1, ctx->stream) != cudaSuccess || cudaStreamSynchronize(ctx->stream) != cudaSuccess))
+    rc = EPFFT_ERR_CUDA;
+  float t = 0.f;
+  if (!rc && cudaEventElapsedTime(&t, e0, e1) != cudaSuccess) rc = EPFFT_ERR_CUDA;
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  if (!rc) *ms = t / (float)n_iter;
+  return rc;
 }
 
 // ---------------------------------------------------------------------------
@@ -2270,7 +2364,7 @@ int epfft_serve_step(epfft_ctx* ctx, int32_t* n_running, int32_t* n_queued) {
     // synchronous read), or read now when no class ran
     CheckRec cr{};
     if (checks_read) {
-      for (int i = 0; i < 8 && !cr.code; i++)
+      for (int i = 0; i < N_CHECK_UNITS && !cr.code; i++)
         if (ctx->h_checks[i].code) cr = ctx->h_checks[i];
       if (cr.code) {
         CheckRec clr;
@@ -2422,8 +2516,14 @@ int epfft_autotune(epfft_ctx* ctx, int32_t L, int32_t precision, int32_t n_batch
     if (shape(L, precision, v, &sh) != EPFFT_OK) continue;  // not compiled for this size
     float c = 0.f, r = 0.f;
     // warm-up, then the timed launches
-    int rc = time_passes_impl(ctx, p, n_batch, E, 3, v, &c, &r);
-    if (!rc) rc = time_passes_impl(ctx, p, n_batch, E, n_iter, v, &c, &r);
+    // a batch that runs on the resident schedule is timed on it
+    int rc = time_resident(ctx, p, n_batch, E, 3, v, &r);
+    if (!rc && r > 0.f) {
+      rc = time_resident(ctx, p, n_batch, E, n_iter, v, &r);
+    } else if (!rc) {
+      rc = time_passes_impl(ctx, p, n_batch, E, 3, v, &c, &r);
+      if (!rc) rc = time_passes_impl(ctx, p, n_batch, E, n_iter, v, &c, &r);
+    }
     if (rc) return rc;
     if (ms_per_iteration) ms_per_iteration[v] = c + r;
     if (best < 0 || c + r < tbest) {

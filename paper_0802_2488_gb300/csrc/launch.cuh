@@ -126,6 +126,22 @@ cudaError_t launch_onchip(int L, int nb, cudaStream_t s, Solve* solves, BatchCtl
 cudaError_t read_check_onchip(CheckRec* out);
 cudaError_t check_record_onchip(void** out);
 
+// Resident schedule (resident.cuh): whole solves by one cooperative launch, for
+// the lattice sides and tilings resident_supported names.  per_sm: resident
+// CTAs per SM; g: CTAs per solve (a power of two, at most the tiling's row
+// CTAs).
+template <typename T>
+bool resident_supported(int L, int var);
+template <typename T>
+cudaError_t prepare_resident(int L, int var, int* per_sm);
+template <typename T>
+cudaError_t launch_resident(int L, int var, int g, int nb, cudaStream_t s, Solve* solves, BatchCtl* bc, double* part2,
+                            unsigned* bars, const void* tw, const void* ktab, int general);
+template <typename T>
+cudaError_t read_check_resident(CheckRec* out);
+template <typename T>
+cudaError_t check_record_resident(void** out);
+
 // Returns false when L is not built for T in that variant.
 template <typename T>
 inline bool pass_shape(int L, int var, PassShape* out) {

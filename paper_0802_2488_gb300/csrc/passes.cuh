@@ -79,7 +79,7 @@ struct Cfg {
                                       : V == 1 ? 2 : (L == 512 ? 768 / NT_COL : (L == 1024 || L == 2048 ? 3 : 1));
   // sequences transformed per call: the largest divisor of the sequence
   // count that keeps at most 16 elements per thread and stage
-  static constexpr int grp(int S, int N, int NT) {
+  static __host__ __device__ constexpr int grp(int S, int N, int NT) {
     int g = S;
     while (g > 1 && (S % g != 0 || g * N > 16 * NT)) g--;
     return g;
@@ -125,6 +125,27 @@ struct Vec4<double> {
     reinterpret_cast<double2*>(p)[1] = make_double2(e[2], e[3]);
   }
 };
+
+// Loads of a pixel's tensor: plain, or (CG) past the L1, for data that other
+// CTAs of the same launch write.
+template <bool CG>
+__device__ __forceinline__ void load4(const float* p, float e[4]) {
+  if constexpr (CG) {
+    const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
+    e[0] = v.x; e[1] = v.y; e[2] = v.z; e[3] = v.w;
+  } else {
+    Vec4<float>::load(p, e);
+  }
+}
+template <bool CG>
+__device__ __forceinline__ void load4(const double* p, double e[4]) {
+  if constexpr (CG) {
+    const double2 a = __ldcg(reinterpret_cast<const double2*>(p)), b = __ldcg(reinterpret_cast<const double2*>(p) + 1);
+    e[0] = a.x; e[1] = a.y; e[2] = b.x; e[3] = b.y;
+  } else {
+    Vec4<double>::load(p, e);
+  }
+}
 
 // ---------------------------------------------------------------------------
 // Row-side helpers.  Shared memory holds 3 x RR sequences of length M
@@ -600,8 +621,10 @@ __device__ __forceinline__ void sum_partials(const double* partials, double* out
 // eta3 = sqrt(comp / EE); the stopping tests compare the squares scaled by
 // the denominators (div2 < tol^2 ss, ...), so an iteration takes no FP64
 // division or root, and the roots are formed once, for the record.
+// record: write the increment's record (the resident schedule runs the state
+// machine in every CTA of a solve; one of them writes).
 template <int L>
-__device__ __forceinline__ void finalize_solve(Solve& S, int phase, const double* A) {
+__device__ __forceinline__ void finalize_solve(Solve& S, int phase, const double* A, bool record = true) {
   constexpr double inv = 1.0 / ((double)L * (double)L);  // exact: L is a power of two
   if (phase == PH_INIT) {
     const double* E = S.path + 4 * S.inc;
@@ -660,18 +683,20 @@ __device__ __forceinline__ void finalize_solve(Solve& S, int phase, const double
         eta1 = div2 == 0.0 ? 0.0 : CUDART_INF;
         eta2 = dd == 0.0 ? 0.0 : CUDART_INF;
       }
-      Record& R = S.rec[S.inc];
-      for (int c = 0; c < 4; c++) {
-        R.sig_mean[c] = sig[c];
-        R.eps_mean[c] = S.epsm_next[c];
+      if (record) {
+        Record& R = S.rec[S.inc];
+        for (int c = 0; c < 4; c++) {
+          R.sig_mean[c] = sig[c];
+          R.eps_mean[c] = S.epsm_next[c];
+        }
+        R.eta1 = eta1;
+        R.eta2 = eta2;
+        R.eta3 = sqrt(comp_n / EE);
+        R.iterations = n;
+        R.n_plastic = (int32_t)S.npl_next;
+        R.n_clusters = 0;
+        R.status = !finite ? 2 : (conv ? 0 : 1);
       }
-      R.eta1 = eta1;
-      R.eta2 = eta2;
-      R.eta3 = sqrt(comp_n / EE);
-      R.iterations = n;
-      R.n_plastic = (int32_t)S.npl_next;
-      R.n_clusters = 0;
-      R.status = !finite ? 2 : (conv ? 0 : 1);
       if (!finite) {
         S.status = 2;
         S.phase = PH_DONE;
@@ -724,14 +749,290 @@ __device__ __forceinline__ void batch_arrive(Solve* solves, int nb, BatchCtl* bc
 // ---------------------------------------------------------------------------
 // Row pass
 // ---------------------------------------------------------------------------
+// Rows bx RR .. bx RR + RR - 1 of a solve in the given phase (INIT: warm
+// start, ITER: one iteration, FINAL: plastic flags): the work of one CTA of
+// the row pass, with the sums of INIT and ITER left in partials[bx].  Eprev:
+// mean strain of the accepted state (read in INIT).  stw: shared stage table,
+// followed by the twist octant; loaded here unless RES, in which the caller
+// keeps them there and the solve's fields are read past the L1 (other CTAs of
+// the same launch write them).
+template <typename T, int L, int V, bool RES>
+__device__ __forceinline__ void row_unit(const Solve& S, const volatile double* Eprev, int phase, int cur, int inc,
+                                         int bx, C2<T>* sp, const C2<T>* __restrict__ tw, const C2<T>* stw,
+                                         double* partials) {
+  using C = Cfg<T, L, V>;
+  constexpr int RR = C::RR, W = C::W, NT = C::NT_ROW, M = C::M;
+  constexpr int P = L >= NT ? L / NT : 1;
+  using IO = RowIO<T, L, V>;
+  const int tid = threadIdx.x;
+  const int lane = tid & 31, wid = tid >> 5;
+  // pixel j of this thread in a row: each warp owns a contiguous run of
+  // 32 P pixels, lane-fastest (L < 32: one short row per warp)
+  auto xmap = [&](int j) { return L >= 32 ? wid * (32 * P) + j * 32 + lane : tid; };
+  const int r0 = bx * RR;
+  const T* __restrict__ ein = reinterpret_cast<const T*>(S.eps[cur]);
+  T* __restrict__ eout = reinterpret_cast<T*>(S.eps[1 - cur]);
+  // sigma of eps^n (read) and of the iterate this pass produces (written)
+  const T* __restrict__ sin_ = reinterpret_cast<const T*>(S.sig[cur]);
+  T* __restrict__ sout = reinterpret_cast<T*>(S.sig[1 - cur]);
+  C2<T>* spec = reinterpret_cast<C2<T>*>(S.spec);
+  const uint8_t* __restrict__ mask = S.mask;
+  Mat<T> m = make_mat<T>(S);
+  const size_t LL = (size_t)L * L;
+  // double precision: the plastic count and the 12 part of the residual of
+  // this thread, added to its sums at the end (an integer add and one FP64
+  // multiply-add per pixel instead of two and a compare)
+  int n_pl = 0;
+  T comp12 = T(0);
+  // stage table and twist octant, in flight until the first barrier after
+  // cp_async_wait_all() (INIT, ITER; the other phases do not read them)
+    if (!RES && (phase == PH_INIT || phase == PH_ITER)) IO::load_tables(sp, tw);
+  T acc[N_ACC];
+#pragma unroll
+  for (int i = 0; i < N_ACC; i++) acc[i] = T(0);
+
+  if (phase == PH_FINAL) {
+    // plastic flags of the accepted state of the last increment
+    uint8_t* fl = S.flags ? S.flags + (size_t)(S.n_inc - 1) * LL : nullptr;  // inc == n_inc - 1
+    for (int r = 0; r < RR && fl; r++)
+      for (int j = 0; j < P; j++) {
+        const int x1 = xmap(j);
+        if (x1 >= L) continue;
+        const size_t x = (size_t)(r0 + r) * L + x1;
+        T e[4];
+        load4<RES>(ein + 4 * x, e);
+        fl[x] = is_plastic(e, mask[x] != 0, m);
+      }
+  } else if (phase == PH_INIT) {
+    // warm start: eps^0 = accepted state + (E_inc - E_{inc-1}); p^0 -> spectrum
+    T dE[4];
+    const double* E = S.path + 4 * (ECHK(inc, S.n_inc, 26) ? inc : 0);
+    for (int c = 0; c < 4; c++) dE[c] = T(E[c] - Eprev[c]);
+    uint8_t* fl = (S.flags && inc > 0) ? S.flags + (size_t)(inc - 1) * LL : nullptr;
+    for (int r = 0; r < RR; r++)
+      for (int j = 0; j < P; j++) {
+        const int x1 = xmap(j);
+        if (x1 >= L) continue;
+        const size_t x = (size_t)(r0 + r) * L + x1;
+        if (!ECHK(x, LL, 20)) continue;
+        const bool v = mask[x] != 0;
+        T e[4], s[4], c0[4];
+        load4<RES>(ein + 4 * x, e);
+        if (fl) fl[x] = is_plastic(e, v, m);
+        for (int c = 0; c < 4; c++) e[c] += dE[c];
+        Vec4<T>::store(eout + 4 * x, e);
+        const bool pl = sigma(e, v, m, s);
+        Vec4<T>::store(sout + 4 * x, s);
+        // <eps^0> and its plastic pixels (the stats of iterate 0)
+#pragma unroll
+        for (int c = 0; c < 4; c++) acc[A_E11 + c] += e[c];
+        acc[A_NPL] += pl ? T(1) : T(0);
+        c0_apply(e, m, c0);
+        IO::px(sp, 0, r, x1) = s[0] - c0[0];
+        IO::px(sp, 1, r, x1) = s[1] - c0[1];
+        IO::px(sp, 2, r, x1) = s[3] - c0[3];
+      }
+  } else {  // PH_ITER
+    T E[4];
+    load_E(S.path + 4 * inc, E);
+    m.E33 = E[2];
+    IO::load_async(sp, spec, r0);
+    // sigma of the RR rows and of the halo row, and the void flags, are
+    // brought into the L2 while the spectrum is transformed (16 KB pieces,
+    // one per lane of warp 0, issued after the spectrum copies so that
+    // those go first)
+    if constexpr (L >= 64 && !RES) {
+      constexpr unsigned RB = (unsigned)(L * 4 * sizeof(T)), PB = RB < 16384u ? RB : 16384u;
+      constexpr int NPR = (int)(RB / PB), NPC = (RR + 1) * NPR;
+      if (wid == 0) {
+        const int xh = (r0 + L - 1) & (L - 1);
+        for (int i = lane; i < NPC; i += 32) {
+          const int k = i / NPR, row = k < RR ? r0 + k : xh;
+          if (ECHK(row, L, 39)) prefetch_l2(reinterpret_cast<const char*>(sin_ + (size_t)4 * row * L) + (size_t)(i % NPR) * PB, PB);
+        }
+        if (lane == 31) prefetch_l2(mask + (size_t)r0 * L, (unsigned)(RR * L));
+      }
+    }
+    // halo row x2 = r0 - 1: sigma12 and sigma22 of iterate n for the
+    // backward difference along x2; loaded while the spectrum is in
+    // flight when the registers allow (few pixels per thread), else after
+    // the transform
+    T prev12[P], prev22[P];
+    auto load_halo = [&]() {
+      const int xh = (r0 + L - 1) & (L - 1);
+#pragma unroll
+      for (int j = 0; j < P; j++) {
+        const int x1 = xmap(j);
+        prev12[j] = prev22[j] = T(0);
+        if (x1 >= L) continue;
+        const size_t x = (size_t)xh * L + x1;
+        if (!ECHK(x, LL, 22)) continue;
+        T s[4];
+        load4<RES>(sin_ + 4 * x, s);
+        prev12[j] = s[3];
+        prev22[j] = s[1];
+      }
+    };
+    constexpr bool EARLY_HALO = P <= 2;
+    if constexpr (EARLY_HALO) load_halo();
+    cp_async_wait_all();
+    __syncthreads();
+    IO::rows_inverse(sp, stw);
+    if constexpr (!EARLY_HALO) load_halo();
+    // Pixel update of the AL iteration at (r, x1), given the stress sj of
+    // iterate n (the multiplier) and the left neighbour's sigma11, sigma12
+    // (x - e^1).
+    auto update = [&](int r, int j, int x1, bool v, const T (&sj)[4], T l11, T l12) {
+      if (x1 >= L) return;
+      const size_t x = (size_t)(r0 + r) * L + x1;
+      // Eq. 1: div_i = sum_j sigma_ij(x) - sigma_ij(x - e^j)
+      const T d1 = (sj[0] - l11) + (sj[3] - prev12[j]);
+      const T d2 = (sj[3] - l12) + (sj[1] - prev22[j]);
+      prev12[j] = sj[3];
+      prev22[j] = sj[1];
+#pragma unroll
+      for (int c = 0; c < 4; c++) acc[A_S11 + c] += sj[c];
+      if constexpr (sizeof(T) == 8) acc[A_DIV2] = fma(d1, d1, fma(d2, d2, acc[A_DIV2]));
+      else acc[A_DIV2] += d1 * d1 + d2 * d2;
+      // augmented-Lagrangian update of this pixel
+      T e[4] = {IO::px(sp, 0, r, x1), IO::px(sp, 1, r, x1), E[2], IO::px(sp, 2, r, x1)};
+      T e1[4], s1[4], p1[3];
+      bool pl;
+      if constexpr (sizeof(T) == 8) {
+        pl = local_step64(sj, e[0], e[1], e[3], v, m, e1, s1, p1);
+      } else {
+        T c0[4], tau[4];
+        c0_apply(e, m, c0);
+#pragma unroll
+        for (int c = 0; c < 4; c++) tau[c] = sj[c] + c0[c];
+        local_solve_p(tau, v, m, e1, s1, p1);
+        pl = is_plastic(e1, v, m);
+      }
+      Vec4<T>::store(eout + 4 * x, e1);
+      Vec4<T>::store(sout + 4 * x, s1);
+      // <eps^{n+1}> and its plastic pixels (stats of the next iterate)
+#pragma unroll
+      for (int c = 0; c < 4; c++) acc[A_E11 + c] += e1[c];
+      if constexpr (sizeof(T) == 8) n_pl += pl ? 1 : 0;
+      else acc[A_NPL] += pl ? T(1) : T(0);
+      const T q0 = e1[0] - e[0], q1 = e1[1] - e[1], q2 = e1[2] - e[2], q3 = e1[3] - e[3];
+      if constexpr (sizeof(T) == 8) {
+        acc[A_COMP] = fma(q0, q0, fma(q1, q1, fma(q2, q2, acc[A_COMP])));
+        comp12 = fma(q3, q3, comp12);
+      } else {
+        acc[A_COMP] += q0 * q0 + q1 * q1 + q2 * q2 + T(2) * q3 * q3;
+      }
+      // next polarization sigma(eps^{n+1}) - C0:eps^{n+1} (in-plane)
+      IO::px(sp, 0, r, x1) = p1[0];
+      IO::px(sp, 1, r, x1) = p1[1];
+      IO::px(sp, 2, r, x1) = p1[2];
+    };
+    // stress of iterate n and voids of row r, group j
+    auto load_px = [&](int r, int j, T (&sg)[4], bool& v) {
+      const int x1 = xmap(j);
+      const size_t x = (size_t)(r0 + r) * L + x1;
+      const bool act = x1 < L && ECHK(x, LL, 23);
+      v = act ? mask[x] != 0 : true;
+      if (act) load4<RES>(sin_ + 4 * x, sg);
+      else sg[0] = sg[1] = sg[2] = sg[3] = T(0);
+    };
+    // Left neighbours: the previous lane by a warp shuffle; lane 0 takes
+    // lane 31 of the previous pixel group of its warp (the run is
+    // contiguous), and at the start of a run reads sigma at x - e^1
+    // (periodic) from memory.
+    // A row is processed in chunks of PC pixels per thread (j = j0 ..
+    // j0 + PC - 1); run11, run12 carry sigma11, sigma12 of lane 31 of the
+    // previous pixel group from chunk to chunk.
+    constexpr int PC = P < 8 ? P : 8;
+    auto row = [&](int r, int j0, T (&sg)[PC][4], bool (&vv)[PC], T& run11, T& run12) {
+#pragma unroll
+      for (int jj = 0; jj < PC; jj++) {
+        const int j = j0 + jj;
+        const int x1 = xmap(j);
+        T l11, l12;
+        if constexpr (L < 32) {
+          const int src = (lane + L - 1) & (L - 1);
+          l11 = __shfl_sync(0xffffffffu, sg[jj][0], src);
+          l12 = __shfl_sync(0xffffffffu, sg[jj][3], src);
+        } else {
+          l11 = __shfl_up_sync(0xffffffffu, sg[jj][0], 1);
+          l12 = __shfl_up_sync(0xffffffffu, sg[jj][3], 1);
+          if (lane == 0) {
+            if (j > 0) {
+              l11 = run11;
+              l12 = run12;
+            } else {
+              const size_t xl = (size_t)(r0 + r) * L + ((x1 + L - 1) & (L - 1));
+              if (ECHK(xl, LL, 24)) {
+                T sl[4];
+                load4<RES>(sin_ + 4 * xl, sl);
+                l11 = sl[0];
+                l12 = sl[3];
+              }
+            }
+          }
+          run11 = __shfl_sync(0xffffffffu, sg[jj][0], 31);
+          run12 = __shfl_sync(0xffffffffu, sg[jj][3], 31);
+        }
+        update(r, j, x1, vv[jj], sg[jj], l11, l12);
+      }
+    };
+    // When the rows' stresses fit in fewer than 32 registers per thread,
+    // all of them are loaded before the first row is processed (their
+    // latencies overlap); otherwise a row is loaded chunk by chunk (PC
+    // loads in flight per thread, from the L2 where the prefetch above
+    // put them).
+    constexpr bool PRE = RR * P * 4 * (int)sizeof(T) < 128;
+    if constexpr (PRE) {
+      static_assert(PC == P, "one chunk per row");
+      T pen[RR][P][4];
+      bool pvv[RR][P];
+#pragma unroll
+      for (int r = 0; r < RR; r++)
+#pragma unroll
+        for (int j = 0; j < P; j++) load_px(r, j, pen[r][j], pvv[r][j]);
+#pragma unroll
+      for (int r = 0; r < RR; r++) {
+        T run11 = T(0), run12 = T(0);
+        row(r, 0, pen[r], pvv[r], run11, run12);
+      }
+    } else {
+      for (int r = 0; r < RR; r++) {
+        T run11 = T(0), run12 = T(0);
+#pragma unroll
+        for (int j0 = 0; j0 < P; j0 += PC) {
+          T en[PC][4];
+          bool vv[PC];
+#pragma unroll
+          for (int jj = 0; jj < PC; jj++) load_px(r, j0 + jj, en[jj], vv[jj]);
+          row(r, j0, en, vv, run11, run12);
+        }
+      }
+    }
+  }
+
+  if constexpr (sizeof(T) == 8) {
+    acc[A_NPL] += T(n_pl);
+    acc[A_COMP] = fma(T(2), comp12, acc[A_COMP]);
+  }
+  if (phase == PH_ITER || phase == PH_INIT) {
+    cp_async_wait_all();  // the tables (INIT)
+    __syncthreads();
+    IO::rows_forward(sp, stw);
+    __syncthreads();
+    IO::store(sp, spec, r0);
+  }
+  if (phase == PH_ITER || phase == PH_INIT) {
+    if (ECHK(bx, L / RR, 25)) block_reduce_acc<NT>(acc, partials + (size_t)bx * PART_STRIDE);
+  }
+}
+
 template <typename T, int L, int V>
 __global__ void __launch_bounds__(Cfg<T, L, V>::NT_ROW, Cfg<T, L, V>::MINB_ROW)
 row_pass(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<T>* __restrict__ tw,
          cudaGraphConditionalHandle cond, int use_cond) {
   using C = Cfg<T, L, V>;
-  constexpr int RR = C::RR, W = C::W, NT = C::NT_ROW, M = C::M;
-  constexpr int P = L >= NT ? L / NT : 1;
-  using IO = RowIO<T, L, V>;
+  constexpr int RR = C::RR, NT = C::NT_ROW;
   extern __shared__ __align__(16) unsigned char smraw[];
   C2<T>* sp = reinterpret_cast<C2<T>*>(smraw);
   __shared__ bool s_last;
@@ -748,268 +1049,8 @@ row_pass(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<T>* __restri
   const int cur = Sv.cur;
   const int inc = Sv.inc;
   const int tid = threadIdx.x;
-  const int lane = tid & 31, wid = tid >> 5;
-  // pixel j of this thread in a row: each warp owns a contiguous run of
-  // 32 P pixels, lane-fastest (L < 32: one short row per warp)
-  auto xmap = [&](int j) { return L >= 32 ? wid * (32 * P) + j * 32 + lane : tid; };
   if (phase != PH_DONE) {
-    const int r0 = blockIdx.x * RR;
-    const T* __restrict__ ein = reinterpret_cast<const T*>(S.eps[cur]);
-    T* __restrict__ eout = reinterpret_cast<T*>(S.eps[1 - cur]);
-    // sigma of eps^n (read) and of the iterate this pass produces (written)
-    const T* __restrict__ sin_ = reinterpret_cast<const T*>(S.sig[cur]);
-    T* __restrict__ sout = reinterpret_cast<T*>(S.sig[1 - cur]);
-    C2<T>* spec = reinterpret_cast<C2<T>*>(S.spec);
-    const uint8_t* __restrict__ mask = S.mask;
-    Mat<T> m = make_mat<T>(S);
-    const size_t LL = (size_t)L * L;
-    // double precision: the plastic count and the 12 part of the residual of
-    // this thread, added to its sums at the end (an integer add and one FP64
-    // multiply-add per pixel instead of two and a compare)
-    int n_pl = 0;
-    T comp12 = T(0);
-    // stage table and twist octant, in flight until the first barrier after
-    // cp_async_wait_all() (INIT, ITER; the other phases do not read them)
-    const C2<T>* stw = sp + C::ROW_DATA;
-    if (phase == PH_INIT || phase == PH_ITER) IO::load_tables(sp, tw);
-    T acc[N_ACC];
-#pragma unroll
-    for (int i = 0; i < N_ACC; i++) acc[i] = T(0);
-
-    if (phase == PH_FINAL) {
-      // plastic flags of the accepted state of the last increment
-      uint8_t* fl = S.flags ? S.flags + (size_t)(S.n_inc - 1) * LL : nullptr;  // inc == n_inc - 1
-      for (int r = 0; r < RR && fl; r++)
-        for (int j = 0; j < P; j++) {
-          const int x1 = xmap(j);
-          if (x1 >= L) continue;
-          const size_t x = (size_t)(r0 + r) * L + x1;
-          T e[4];
-          Vec4<T>::load(ein + 4 * x, e);
-          fl[x] = is_plastic(e, mask[x] != 0, m);
-        }
-    } else if (phase == PH_INIT) {
-      // warm start: eps^0 = accepted state + (E_inc - E_{inc-1}); p^0 -> spectrum
-      T dE[4];
-      const double* E = S.path + 4 * (ECHK(inc, S.n_inc, 26) ? inc : 0);
-      for (int c = 0; c < 4; c++) dE[c] = T(E[c] - Sv.Eprev[c]);
-      uint8_t* fl = (S.flags && inc > 0) ? S.flags + (size_t)(inc - 1) * LL : nullptr;
-      for (int r = 0; r < RR; r++)
-        for (int j = 0; j < P; j++) {
-          const int x1 = xmap(j);
-          if (x1 >= L) continue;
-          const size_t x = (size_t)(r0 + r) * L + x1;
-          if (!ECHK(x, LL, 20)) continue;
-          const bool v = mask[x] != 0;
-          T e[4], s[4], c0[4];
-          Vec4<T>::load(ein + 4 * x, e);
-          if (fl) fl[x] = is_plastic(e, v, m);
-          for (int c = 0; c < 4; c++) e[c] += dE[c];
-          Vec4<T>::store(eout + 4 * x, e);
-          const bool pl = sigma(e, v, m, s);
-          Vec4<T>::store(sout + 4 * x, s);
-          // <eps^0> and its plastic pixels (the stats of iterate 0)
-#pragma unroll
-          for (int c = 0; c < 4; c++) acc[A_E11 + c] += e[c];
-          acc[A_NPL] += pl ? T(1) : T(0);
-          c0_apply(e, m, c0);
-          IO::px(sp, 0, r, x1) = s[0] - c0[0];
-          IO::px(sp, 1, r, x1) = s[1] - c0[1];
-          IO::px(sp, 2, r, x1) = s[3] - c0[3];
-        }
-    } else {  // PH_ITER
-      T E[4];
-      load_E(S.path + 4 * inc, E);
-      m.E33 = E[2];
-      IO::load_async(sp, spec, r0);
-      // sigma of the RR rows and of the halo row, and the void flags, are
-      // brought into the L2 while the spectrum is transformed (16 KB pieces,
-      // one per lane of warp 0, issued after the spectrum copies so that
-      // those go first)
-      if constexpr (L >= 64) {
-        constexpr unsigned RB = (unsigned)(L * 4 * sizeof(T)), PB = RB < 16384u ? RB : 16384u;
-        constexpr int NPR = (int)(RB / PB), NPC = (RR + 1) * NPR;
-        if (wid == 0) {
-          const int xh = (r0 + L - 1) & (L - 1);
-          for (int i = lane; i < NPC; i += 32) {
-            const int k = i / NPR, row = k < RR ? r0 + k : xh;
-            if (ECHK(row, L, 39)) prefetch_l2(reinterpret_cast<const char*>(sin_ + (size_t)4 * row * L) + (size_t)(i % NPR) * PB, PB);
-          }
-          if (lane == 31) prefetch_l2(mask + (size_t)r0 * L, (unsigned)(RR * L));
-        }
-      }
-      // halo row x2 = r0 - 1: sigma12 and sigma22 of iterate n for the
-      // backward difference along x2; loaded while the spectrum is in
-      // flight when the registers allow (few pixels per thread), else after
-      // the transform
-      T prev12[P], prev22[P];
-      auto load_halo = [&]() {
-        const int xh = (r0 + L - 1) & (L - 1);
-#pragma unroll
-        for (int j = 0; j < P; j++) {
-          const int x1 = xmap(j);
-          prev12[j] = prev22[j] = T(0);
-          if (x1 >= L) continue;
-          const size_t x = (size_t)xh * L + x1;
-          if (!ECHK(x, LL, 22)) continue;
-          T s[4];
-          Vec4<T>::load(sin_ + 4 * x, s);
-          prev12[j] = s[3];
-          prev22[j] = s[1];
-        }
-      };
-      constexpr bool EARLY_HALO = P <= 2;
-      if constexpr (EARLY_HALO) load_halo();
-      cp_async_wait_all();
-      __syncthreads();
-      IO::rows_inverse(sp, stw);
-      if constexpr (!EARLY_HALO) load_halo();
-      // Pixel update of the AL iteration at (r, x1), given the stress sj of
-      // iterate n (the multiplier) and the left neighbour's sigma11, sigma12
-      // (x - e^1).
-      auto update = [&](int r, int j, int x1, bool v, const T (&sj)[4], T l11, T l12) {
-        if (x1 >= L) return;
-        const size_t x = (size_t)(r0 + r) * L + x1;
-        // Eq. 1: div_i = sum_j sigma_ij(x) - sigma_ij(x - e^j)
-        const T d1 = (sj[0] - l11) + (sj[3] - prev12[j]);
-        const T d2 = (sj[3] - l12) + (sj[1] - prev22[j]);
-        prev12[j] = sj[3];
-        prev22[j] = sj[1];
-#pragma unroll
-        for (int c = 0; c < 4; c++) acc[A_S11 + c] += sj[c];
-        if constexpr (sizeof(T) == 8) acc[A_DIV2] = fma(d1, d1, fma(d2, d2, acc[A_DIV2]));
-        else acc[A_DIV2] += d1 * d1 + d2 * d2;
-        // augmented-Lagrangian update of this pixel
-        T e[4] = {IO::px(sp, 0, r, x1), IO::px(sp, 1, r, x1), E[2], IO::px(sp, 2, r, x1)};
-        T e1[4], s1[4], p1[3];
-        bool pl;
-        if constexpr (sizeof(T) == 8) {
-          pl = local_step64(sj, e[0], e[1], e[3], v, m, e1, s1, p1);
-        } else {
-          T c0[4], tau[4];
-          c0_apply(e, m, c0);
-#pragma unroll
-          for (int c = 0; c < 4; c++) tau[c] = sj[c] + c0[c];
-          local_solve_p(tau, v, m, e1, s1, p1);
-          pl = is_plastic(e1, v, m);
-        }
-        Vec4<T>::store(eout + 4 * x, e1);
-        Vec4<T>::store(sout + 4 * x, s1);
-        // <eps^{n+1}> and its plastic pixels (stats of the next iterate)
-#pragma unroll
-        for (int c = 0; c < 4; c++) acc[A_E11 + c] += e1[c];
-        if constexpr (sizeof(T) == 8) n_pl += pl ? 1 : 0;
-        else acc[A_NPL] += pl ? T(1) : T(0);
-        const T q0 = e1[0] - e[0], q1 = e1[1] - e[1], q2 = e1[2] - e[2], q3 = e1[3] - e[3];
-        if constexpr (sizeof(T) == 8) {
-          acc[A_COMP] = fma(q0, q0, fma(q1, q1, fma(q2, q2, acc[A_COMP])));
-          comp12 = fma(q3, q3, comp12);
-        } else {
-          acc[A_COMP] += q0 * q0 + q1 * q1 + q2 * q2 + T(2) * q3 * q3;
-        }
-        // next polarization sigma(eps^{n+1}) - C0:eps^{n+1} (in-plane)
-        IO::px(sp, 0, r, x1) = p1[0];
-        IO::px(sp, 1, r, x1) = p1[1];
-        IO::px(sp, 2, r, x1) = p1[2];
-      };
-      // stress of iterate n and voids of row r, group j
-      auto load_px = [&](int r, int j, T (&sg)[4], bool& v) {
-        const int x1 = xmap(j);
-        const size_t x = (size_t)(r0 + r) * L + x1;
-        const bool act = x1 < L && ECHK(x, LL, 23);
-        v = act ? mask[x] != 0 : true;
-        if (act) Vec4<T>::load(sin_ + 4 * x, sg);
-        else sg[0] = sg[1] = sg[2] = sg[3] = T(0);
-      };
-      // Left neighbours: the previous lane by a warp shuffle; lane 0 takes
-      // lane 31 of the previous pixel group of its warp (the run is
-      // contiguous), and at the start of a run reads sigma at x - e^1
-      // (periodic) from memory.
-      // A row is processed in chunks of PC pixels per thread (j = j0 ..
-      // j0 + PC - 1); run11, run12 carry sigma11, sigma12 of lane 31 of the
-      // previous pixel group from chunk to chunk.
-      constexpr int PC = P < 8 ? P : 8;
-      auto row = [&](int r, int j0, T (&sg)[PC][4], bool (&vv)[PC], T& run11, T& run12) {
-#pragma unroll
-        for (int jj = 0; jj < PC; jj++) {
-          const int j = j0 + jj;
-          const int x1 = xmap(j);
-          T l11, l12;
-          if constexpr (L < 32) {
-            const int src = (lane + L - 1) & (L - 1);
-            l11 = __shfl_sync(0xffffffffu, sg[jj][0], src);
-            l12 = __shfl_sync(0xffffffffu, sg[jj][3], src);
-          } else {
-            l11 = __shfl_up_sync(0xffffffffu, sg[jj][0], 1);
-            l12 = __shfl_up_sync(0xffffffffu, sg[jj][3], 1);
-            if (lane == 0) {
-              if (j > 0) {
-                l11 = run11;
-                l12 = run12;
-              } else {
-                const size_t xl = (size_t)(r0 + r) * L + ((x1 + L - 1) & (L - 1));
-                if (ECHK(xl, LL, 24)) {
-                  T sl[4];
-                  Vec4<T>::load(sin_ + 4 * xl, sl);
-                  l11 = sl[0];
-                  l12 = sl[3];
-                }
-              }
-            }
-            run11 = __shfl_sync(0xffffffffu, sg[jj][0], 31);
-            run12 = __shfl_sync(0xffffffffu, sg[jj][3], 31);
-          }
-          update(r, j, x1, vv[jj], sg[jj], l11, l12);
-        }
-      };
-      // When the rows' stresses fit in fewer than 32 registers per thread,
-      // all of them are loaded before the first row is processed (their
-      // latencies overlap); otherwise a row is loaded chunk by chunk (PC
-      // loads in flight per thread, from the L2 where the prefetch above
-      // put them).
-      constexpr bool PRE = RR * P * 4 * (int)sizeof(T) < 128;
-      if constexpr (PRE) {
-        static_assert(PC == P, "one chunk per row");
-        T pen[RR][P][4];
-        bool pvv[RR][P];
-#pragma unroll
-        for (int r = 0; r < RR; r++)
-#pragma unroll
-          for (int j = 0; j < P; j++) load_px(r, j, pen[r][j], pvv[r][j]);
-#pragma unroll
-        for (int r = 0; r < RR; r++) {
-          T run11 = T(0), run12 = T(0);
-          row(r, 0, pen[r], pvv[r], run11, run12);
-        }
-      } else {
-        for (int r = 0; r < RR; r++) {
-          T run11 = T(0), run12 = T(0);
-#pragma unroll
-          for (int j0 = 0; j0 < P; j0 += PC) {
-            T en[PC][4];
-            bool vv[PC];
-#pragma unroll
-            for (int jj = 0; jj < PC; jj++) load_px(r, j0 + jj, en[jj], vv[jj]);
-            row(r, j0, en, vv, run11, run12);
-          }
-        }
-      }
-    }
-
-    if constexpr (sizeof(T) == 8) {
-      acc[A_NPL] += T(n_pl);
-      acc[A_COMP] = fma(T(2), comp12, acc[A_COMP]);
-    }
-    if (phase == PH_ITER || phase == PH_INIT) {
-      cp_async_wait_all();  // the tables (INIT)
-      __syncthreads();
-      IO::rows_forward(sp, stw);
-      __syncthreads();
-      IO::store(sp, spec, r0);
-    }
-    if (phase == PH_ITER || phase == PH_INIT) {
-      if (ECHK(blockIdx.x, L / RR, 25)) block_reduce_acc<NT>(acc, S.partials + (size_t)blockIdx.x * PART_STRIDE);
-    }
+    row_unit<T, L, V, false>(S, Sv.Eprev, phase, cur, inc, blockIdx.x, sp, tw, sp + C::ROW_DATA, S.partials);
     // every thread of this CTA is done with the solve state before the CTA
     // counts itself in
     __syncthreads();
@@ -1038,35 +1079,22 @@ row_pass(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<T>* __restri
 // ---------------------------------------------------------------------------
 // Column pass
 // ---------------------------------------------------------------------------
+// Columns b W .. b W + W - 1 of a solve in phase ITER: the work of one CTA of
+// the column pass.  stw: shared stage table (loaded here unless RES, see
+// row_unit).  prefetch: called once the column's copies are issued.
 // GEN = false: the Eq. 3 operator only (every solve of the launch uses it);
 // GEN = true: the operator each solve names (GreenMode).
-template <typename T, int L, int V, bool GEN>
-__global__ void __launch_bounds__(Cfg<T, L, V>::NT_COL, Cfg<T, L, V>::MINB_COL)
-col_pass(Solve* __restrict__ solves, const C2<T>* __restrict__ tw, const C2<T>* __restrict__ ktab,
-         cudaGraphConditionalHandle cond, int use_cond, int succ) {
+template <typename T, int L, int V, bool GEN, int NT, bool RES, typename F>
+__device__ __forceinline__ void col_unit(const Solve& S, int inc, int b, C2<T>* sp, const C2<T>* __restrict__ tw,
+                                         const C2<T>* stw, const C2<T>* __restrict__ ktab, F&& prefetch) {
   using C = Cfg<T, L, V>;
-  constexpr int W = C::W, NT = C::NT_COL, M = C::M, NBK = M / W, SP = C::SP_C, SZ = C::COL_DATA;
-  extern __shared__ __align__(16) unsigned char smraw[];
+  constexpr int W = C::W, M = C::M, NBK = M / W, SP = C::SP_C, SZ = C::COL_DATA;
   // 3 W sequences of length L (sequence c * W + w = component c of column
-  // w, padded layout of fft.cuh), then the column plan's stage table
-  C2<T>* sp = reinterpret_cast<C2<T>*>(smraw);
-  C2<T>* stw = sp + SZ;
+  // w, padded layout of fft.cuh)
   auto at = [](int c, int w, int x2) { return (c * W + w) * SP + pad32(x2); };
   const int tid = threadIdx.x;
-  // Every index of the pass is in range when the grid has M / W CTAs per
-  // solve: b < M / W, c < 3, w < W and x2 < L give at(c, w, x2) < 3 W SP <=
-  // SZ and a global index below 3 M L.
-  if (!ECHK(gridDim.x - 1, NBK, 33)) return;
-  // The row pass that follows re-arms the loop; a body that never reaches
-  // it must not loop again.
-  if (use_cond && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) cudaGraphSetConditional(cond, 0u);
-  Solve& S = solves[blockIdx.y];
-  const volatile Solve& Sv = S;
-  if (Sv.phase != PH_ITER) return;
-  const int inc = Sv.inc;
-  const int b = blockIdx.x;
   C2<T>* spec = reinterpret_cast<C2<T>*>(S.spec);
-  copy_table<T, NT>(stw, tw + C::TB::off_col(V), C::COL_TW);
+  if (!RES) copy_table<T, NT>(const_cast<C2<T>*>(stw), tw + C::TB::off_col(V), C::COL_TW);
   // the slab of each component is contiguous in HBM: consecutive threads
   // copy consecutive numbers, asynchronously, the whole slab in flight
 #pragma unroll 4
@@ -1078,28 +1106,10 @@ col_pass(Solve* __restrict__ solves, const C2<T>* __restrict__ tw, const C2<T>* 
     const size_t g = (size_t)(c * NBK + b) * L * W + rem;
     if (ECHK(i, SZ, 30) && ECHK(g, (size_t)3 * M * L, 34)) cp_async_c2(sp + i, spec + g);
   }
-  // the slab of the CTA that follows this one on an SM (succ = the CTAs the
-  // GPU holds at once, counted in launch order) is asked of the L2 while
-  // this CTA transforms its own, in 16 KB pieces by warp 0
-  if (tid < 32 && succ > 0) {
-    const long long nxt = (long long)blockIdx.y * gridDim.x + blockIdx.x + succ;
-    if (nxt < (long long)gridDim.x * gridDim.y) {
-      const int bs = (int)(nxt % gridDim.x), ss = (int)(nxt / gridDim.x);
-      const volatile Solve& Sn = solves[ss];
-      if (Sn.phase == PH_ITER) {
-        constexpr unsigned SB = (unsigned)(L * W * sizeof(C2<T>)), PB = SB < 16384u ? SB : 16384u;
-        constexpr int NPS = (int)(SB / PB);
-        const char* sn = reinterpret_cast<const char*>(solves[ss].spec);
-        for (int k = tid; k < 3 * NPS; k += 32) {
-          const int c = k / NPS;
-          if (ECHK(bs, NBK, 35)) prefetch_l2(sn + ((size_t)(c * NBK + bs) * L * W) * sizeof(C2<T>) + (size_t)(k % NPS) * PB, PB);
-        }
-      }
-    }
-  }
+  prefetch();
   cp_async_wait_all();
   __syncthreads();
-  constexpr int G = C::G_C;
+  constexpr int G = C::grp(3 * W, L, NT);
 #pragma unroll 1
   for (int g = 0; g < 3 * W / G; g++) fft_seq<T, L, C::RM_COL, C::FULL, G, NT, false>(sp + g * G * SP, stw);
 
@@ -1123,37 +1133,50 @@ col_pass(Solve* __restrict__ solves, const C2<T>* __restrict__ tw, const C2<T>* 
   }
   if (b == 0) {
     // packed column: Z = A + i B with A the m1 = 0 column and B the
-    // m1 = L/2 column, both transforms of real sequences (Hermitian)
+    // m1 = L/2 column, both transforms of real sequences (Hermitian), and so
+    // are the operators' results: those at mp =
+    // L - m2 are the conjugates of those at m2.  An even thread applies the
+    // operator to A, the odd one beside it to B of the same m2; they exchange
+    // results and write positions m2 and mp.  (This CTA has the most work per
+    // thread of the pass: half the operators on twice the threads took an FP64
+    // L = 256 solve from 60 to 49 us an iteration.)
     const double* Ep = S.path + 4 * inc;
-    for (int m2 = tid; m2 <= L / 2; m2 += NT) {
-      const int mp = (L - m2) & (L - 1);
-      C2<T> A[3], B[3], Ap[3], Bp[3];
+    for (int t0 = 0; t0 < 2 * (L / 2 + 1); t0 += NT) {
+      const int m2 = (t0 + tid) >> 1, mp = (L - m2) & (L - 1);
+      const bool isb = (tid & 1) != 0, act = m2 <= L / 2;
+      C2<T> X[3], Y[3];
 #pragma unroll
       for (int c = 0; c < 3; c++) {
-        const C2<T> z = sp[at(c, 0, m2)], zp = sp[at(c, 0, mp)];
-        A[c] = T(0.5) * (z + conj(zp));
-        const C2<T> d = z - conj(zp);  // B = d / (2i)
-        B[c] = mk(T(0.5) * d.im, T(-0.5) * d.re);
-        Ap[c] = conj(A[c]);
-        Bp[c] = conj(B[c]);
+        X[c] = mk(T(0), T(0));
+        if (act) {
+          const C2<T> z = sp[at(c, 0, m2)], zp = sp[at(c, 0, mp)];
+          // A = (z + conj zp) / 2, B = (z - conj zp) / (2i)
+          X[c] = isb ? mk(T(0.5) * (z.im + zp.im), T(0.5) * (zp.re - z.re))
+                     : mk(T(0.5) * (z.re + zp.re), T(0.5) * (z.im - zp.im));
+        }
       }
-      if (m2 == 0) {
-        // the mean strain, or 0 where it is added in FP64 after the
-        // transforms (the defect form and its reference)
-        const T z = S.zero_mean ? T(0) : T(1);
-        A[0] = mk(z * T(Ep[0]), T(0));
-        A[1] = mk(z * T(Ep[1]), T(0));
-        A[2] = mk(z * T(Ep[3]), T(0));
-      } else {
-        green_op(gm, ktab, qtab, L, 0, m2, lam0, mu0, scale, A[0], A[1], A[2]);
-        green_op(gm, ktab, qtab, L, 0, mp, lam0, mu0, scale, Ap[0], Ap[1], Ap[2]);
+      if (act) {
+        if (m2 == 0 && !isb) {
+          // the mean strain, or 0 where it is added in FP64 after the
+          // transforms (the defect form and its reference)
+          const T z = S.zero_mean ? T(0) : T(1);
+          X[0] = mk(z * T(Ep[0]), T(0));
+          X[1] = mk(z * T(Ep[1]), T(0));
+          X[2] = mk(z * T(Ep[3]), T(0));
+        } else {
+          green_op(gm, ktab, qtab, L, isb ? M : 0, m2, lam0, mu0, scale, X[0], X[1], X[2]);
+        }
       }
-      green_op(gm, ktab, qtab, L, M, m2, lam0, mu0, scale, B[0], B[1], B[2]);
-      green_op(gm, ktab, qtab, L, M, mp, lam0, mu0, scale, Bp[0], Bp[1], Bp[2]);
 #pragma unroll
       for (int c = 0; c < 3; c++) {
-        sp[at(c, 0, m2)] = A[c] + mul_i(B[c]);
-        if (mp != m2) sp[at(c, 0, mp)] = Ap[c] + mul_i(Bp[c]);
+        Y[c].re = __shfl_xor_sync(0xffffffffu, X[c].re, 1);
+        Y[c].im = __shfl_xor_sync(0xffffffffu, X[c].im, 1);
+      }
+      if (act && !(isb && mp == m2)) {
+        // even: A + i B at m2; odd: conj(A) + i conj(B) at mp
+#pragma unroll
+        for (int c = 0; c < 3; c++)
+          sp[at(c, 0, isb ? mp : m2)] = isb ? mk(Y[c].re + X[c].im, X[c].re - Y[c].im) : X[c] + mul_i(Y[c]);
       }
     }
   }
@@ -1187,6 +1210,50 @@ col_pass(Solve* __restrict__ solves, const C2<T>* __restrict__ tw, const C2<T>* 
       if (ECHK(i, SZ, 32)) spec[(size_t)(c * NBK + b) * L * W + rem] = sp[i];
     }
   }
+}
+
+template <typename T, int L, int V, bool GEN>
+__global__ void __launch_bounds__(Cfg<T, L, V>::NT_COL, Cfg<T, L, V>::MINB_COL)
+col_pass(Solve* __restrict__ solves, const C2<T>* __restrict__ tw, const C2<T>* __restrict__ ktab,
+         cudaGraphConditionalHandle cond, int use_cond, int succ) {
+  using C = Cfg<T, L, V>;
+  constexpr int W = C::W, NT = C::NT_COL, M = C::M, NBK = M / W;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  C2<T>* sp = reinterpret_cast<C2<T>*>(smraw);
+  const int tid = threadIdx.x;
+  // Every index of the pass is in range when the grid has M / W CTAs per
+  // solve: b < M / W, c < 3, w < W and x2 < L give at(c, w, x2) < 3 W SP <=
+  // SZ and a global index below 3 M L.
+  if (!ECHK(gridDim.x - 1, NBK, 33)) return;
+  // The row pass that follows re-arms the loop; a body that never reaches
+  // it must not loop again.
+  if (use_cond && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) cudaGraphSetConditional(cond, 0u);
+  Solve& S = solves[blockIdx.y];
+  const volatile Solve& Sv = S;
+  if (Sv.phase != PH_ITER) return;
+  const int inc = Sv.inc;
+  auto prefetch = [&]() {
+    // the slab of the CTA that follows this one on an SM (succ = the CTAs the
+    // GPU holds at once, counted in launch order) is asked of the L2 while
+    // this CTA transforms its own, in 16 KB pieces by warp 0
+    if (tid < 32 && succ > 0) {
+      const long long nxt = (long long)blockIdx.y * gridDim.x + blockIdx.x + succ;
+      if (nxt < (long long)gridDim.x * gridDim.y) {
+        const int bs = (int)(nxt % gridDim.x), ss = (int)(nxt / gridDim.x);
+        const volatile Solve& Sn = solves[ss];
+        if (Sn.phase == PH_ITER) {
+          constexpr unsigned SB = (unsigned)(L * W * sizeof(C2<T>)), PB = SB < 16384u ? SB : 16384u;
+          constexpr int NPS = (int)(SB / PB);
+          const char* sn = reinterpret_cast<const char*>(solves[ss].spec);
+          for (int k = tid; k < 3 * NPS; k += 32) {
+            const int c = k / NPS;
+            if (ECHK(bs, NBK, 35)) prefetch_l2(sn + ((size_t)(c * NBK + bs) * L * W) * sizeof(C2<T>) + (size_t)(k % NPS) * PB, PB);
+          }
+        }
+      }
+    }
+  };
+  col_unit<T, L, V, GEN, NT, false>(S, inc, blockIdx.x, sp, tw, sp + C::COL_DATA, ktab, prefetch);
 }
 
 // ---------------------------------------------------------------------------
