@@ -1118,8 +1118,8 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
     if (streaming > 1) k += steps;  // the loop-condition kernel of the mixed graph
     // the defect form's refreshes: from the host, and the loop body's node
     for (int g = 0; g < G; g++) k += 4 * (Bs[g].refreshes + bc[g].refresh_runs);
-    // per solve the mask kernel (when generated) and the four labelling kernels
-    for (int i = 0; i < n; i++) k += (probs[i].mask ? 0 : 1) + 4;
+    // per solve the mask kernel (when generated) and the three labelling kernels
+    for (int i = 0; i < n; i++) k += (probs[i].mask ? 0 : 1) + 3;
     c->last.loop_steps = steps;
     c->last.kernel_launches = k;
     c->last.iterations = its;
@@ -1814,7 +1814,7 @@ int epfft_solve_dg2(epfft_ctx* ctx, const epfft_problem* problem, const epfft_pa
   for (size_t i = 0; i < LL; i++) npl += hf[i];
   records[n_inc - 1].n_plastic = npl;
   records[n_inc - 1].n_clusters = hc[0];
-  ctx->last.kernel_launches += 3 + (problem->mask ? 0 : 1) + 2 + 4;
+  ctx->last.kernel_launches += 3 + (problem->mask ? 0 : 1) + 2 + 3;
   return status;
 }
 
@@ -1825,39 +1825,51 @@ int epfft_void_plastic(epfft_ctx* ctx, int32_t L, int32_t n_img, const uint8_t* 
   if (cudaSetDevice(ctx->device) != cudaSuccess) return EPFFT_ERR_CUDA;
   const size_t LL = (size_t)L * L;
   Arena A(ctx);
-  uint8_t* vp = (uint8_t*)A.get(LL);
-  int32_t* lab = (int32_t*)A.get(sizeof(int32_t) * LL);
-  int32_t* out = labels_dev ? nullptr : (int32_t*)A.get(sizeof(int32_t) * LL);
-  void* scratch = A.get(22 * LL);
-  int32_t* dcnt = (int32_t*)A.get(8 * sizeof(int32_t));
-  if (!vp || !lab || (!labels_dev && !out) || !scratch || !dcnt) return EPFFT_ERR_OOM;
+  // images at a time: up to 512 MB of labels and scratch, fewer (down to one)
+  // if that cannot be had
+  const size_t per = LL * (sizeof(int32_t) + VP_SCRATCH_BYTES);
+  int64_t step = std::max<int64_t>(1, std::min<int64_t>(n_img, (int64_t)(((size_t)512 << 20) / per)));
+  char* buf = (char*)A.get(per * (size_t)step);
+  if (!buf && step > 1) buf = (char*)A.get(per * (size_t)(step = 1));
+  // counts: 4 per image, then clusters and pixels of the voids, the error flag
+  const size_t ncnt = 4 * (size_t)n_img + 3;
+  int32_t* dcnt = (int32_t*)A.get(ncnt * sizeof(int32_t));
+  if (!buf || !dcnt) return EPFFT_ERR_OOM;
+  int32_t* voids = dcnt + 4 * (size_t)n_img;
+  const size_t m = LL * (size_t)step;
+  VpScratch vp;
+  vp.best = (unsigned long long*)buf;
+  int32_t* lab = (int32_t*)(vp.best + m);
+  vp.target = lab + m;
+  vp.final_root = vp.target + m;
+  vp.size = vp.final_root + m;
+  vp.has_void = (uint8_t*)(vp.size + m);
+  vp.has_pl = vp.has_void + m;
+  CK(cudaMemsetAsync(dcnt, 0, ncnt * sizeof(int32_t), ctx->stream));
   // the voids alone: their clusters and pixels (once)
-  CK(cudaMemsetAsync(dcnt, 0, 8 * sizeof(int32_t), ctx->stream));
-  CK(launch_label(mask_dev, lab, 1, L, 1, dcnt + 3, dcnt + 7, ctx->stream));
-  CK(launch_count(mask_dev, (int64_t)LL, dcnt + 5, ctx->stream));
-  int32_t hv[8];
-  CK(cudaMemcpyAsync(hv, dcnt, sizeof(hv), cudaMemcpyDeviceToHost, ctx->stream));
+  CK(launch_label(mask_dev, lab, 1, L, 1, voids, voids + 2, ctx->stream, false));
+  CK(launch_count(mask_dev, (int64_t)LL, voids + 1, ctx->stream));
+  for (int64_t k = 0; k < n_img; k += step) {
+    const int64_t n = std::min<int64_t>(step, n_img - k);
+    vp.stats = dcnt + 4 * k;
+    CK(launch_vp_label(mask_dev, plastic_dev + (size_t)k * LL, lab, n, L, vp, voids + 2, ctx->stream));
+    CK(launch_vp_attach(mask_dev, lab, labels_dev ? labels_dev + (size_t)k * LL : nullptr, n, L, vp, voids + 1,
+                        ctx->stream));
+  }
+  std::vector<int32_t> h(ncnt);
+  CK(cudaMemcpyAsync(h.data(), dcnt, ncnt * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
-  if (hv[7]) return EPFFT_ERR_DEVICE_TIMEOUT;
+  const int32_t* hv = h.data() + 4 * (size_t)n_img;
+  if (hv[2]) return EPFFT_ERR_DEVICE_TIMEOUT;
   for (int k = 0; k < n_img; k++) {
-    const uint8_t* pl = plastic_dev + (size_t)k * LL;
-    int32_t* o = labels_dev ? labels_dev + (size_t)k * LL : out;
-    CK(cudaMemsetAsync(dcnt, 0, 8 * sizeof(int32_t), ctx->stream));
-    CK(launch_vp_flags(mask_dev, pl, vp, L, ctx->stream));
-    CK(launch_label(vp, lab, 1, L, 1, dcnt + 6, dcnt + 7, ctx->stream));
-    CK(launch_vp_attach(mask_dev, vp, lab, o, L, scratch, dcnt, hv[5] > 0, ctx->stream));
-    CK(launch_count(pl, (int64_t)LL, dcnt + 4, ctx->stream));
-    int32_t h[8];
-    CK(cudaMemcpyAsync(h, dcnt, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    if (h[7]) return EPFFT_ERR_DEVICE_TIMEOUT;
+    const int32_t* d = h.data() + 4 * (size_t)k;
     int32_t* st = stats + 6 * (size_t)k;
-    st[0] = h[0];
-    st[1] = h[1];
-    st[2] = h[2];
-    st[3] = hv[3];
-    st[4] = h[4];
-    st[5] = hv[5];
+    st[0] = d[0];
+    st[1] = d[1];
+    st[2] = d[2];
+    st[3] = hv[0];
+    st[4] = d[3];
+    st[5] = hv[1];
   }
   return EPFFT_OK;
 }
@@ -2385,7 +2397,7 @@ int epfft_serve_step(epfft_ctx* ctx, int32_t* n_running, int32_t* n_queued) {
     rc = serve_harvest(ctx, S, k);
     if (rc) return rc;
     for (auto& sl : k->slots) after += sl.used;
-    ctx->last.kernel_launches += 4 * (before - after);  // labelling of each harvested solve
+    ctx->last.kernel_launches += 3 * (before - after);  // labelling of each harvested solve
   }
   int running = 0;
   for (auto& kv : S.classes)

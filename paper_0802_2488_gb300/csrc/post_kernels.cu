@@ -64,44 +64,23 @@ __global__ void avg5_kernel(const T* __restrict__ in, T* __restrict__ out, int L
 
 // --- Sec. 3: void-plastic clusters with nearest-void attachment ----------
 
-__global__ void vp_flags_kernel(const uint8_t* __restrict__ mask, const uint8_t* __restrict__ pl,
-                                uint8_t* __restrict__ vp, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    vp[i] = (uint8_t)(mask[i] | pl[i]);
-}
-
-// best[] = all ones; final_root[] = n; size[] = 0; has_pl[] = 0
-__global__ void vp_init_kernel(unsigned long long* __restrict__ best, int32_t* __restrict__ final_root,
-                               int32_t* __restrict__ size, uint8_t* __restrict__ has_pl, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    best[i] = ~0ull;
-    final_root[i] = (int32_t)n;
-    size[i] = 0;
-    has_pl[i] = 0;
-  }
-}
-
-// has_void[root] = 1 for clusters holding a void
-__global__ void vp_mark_kernel(const uint8_t* __restrict__ mask, const int32_t* __restrict__ lab,
-                               uint8_t* __restrict__ has_void, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    if (mask[i] && lab[i] >= 0 && lab[i] < n) has_void[lab[i]] = 1;
-}
-
 // Each pixel of a void-free cluster finds its nearest void by Chebyshev
 // rings r = 0, 1, ... (periodic), keeping the smallest (d^2, index); ring
 // r + 1 holds only pixels with d^2 >= (r + 1)^2, so the search stops once
 // that exceeds the best d^2, and at r = L/2 at the latest.  The cluster's
 // minimum is the atomic minimum of the packed key d^2 * 2^32 + index.
-__global__ void vp_nearest_kernel(const uint8_t* __restrict__ mask, const uint8_t* __restrict__ vp,
-                                  const int32_t* __restrict__ lab, const uint8_t* __restrict__ has_void,
-                                  unsigned long long* __restrict__ best, int L) {
+// One mask, n_img images of labels; n_voids: void pixels of the mask (none:
+// nothing to find).
+__global__ void vp_nearest_kernel(const uint8_t* __restrict__ mask, const int32_t* __restrict__ lab, VpScratch vp,
+                                  const int32_t* __restrict__ n_voids, int L, int64_t n_img) {
   const int64_t n = (int64_t)L * L;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    if (!vp[i] || mask[i]) continue;
+  if (*n_voids == 0) return;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n * n_img; i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t root = lab[i];
-    if (root < 0 || root >= n || has_void[root]) continue;
-    const int x1 = (int)(i % L), x2 = (int)(i / L);
+    if (root < 0) continue;
+    const int64_t img = i / n, x0 = i - img * n;
+    if (mask[x0] || vp.has_void[img * n + root]) continue;
+    const int x1 = (int)(x0 % L), x2 = (int)(x0 / L);
     unsigned long long key = ~0ull;
     int64_t bd = -1;
     for (int r = 0; r <= L / 2; r++) {
@@ -126,43 +105,49 @@ __global__ void vp_nearest_kernel(const uint8_t* __restrict__ mask, const uint8_
         }
       }
     }
-    if (key != ~0ull) atomicMin(best + root, key);
+    if (key != ~0ull) atomicMin(vp.best + img * n + root, key);
   }
 }
 
 // target[root]: the root itself, or the root of the cluster of its nearest
 // void; final_root[target] = smallest root merged into it
-__global__ void vp_target_kernel(const uint8_t* __restrict__ vp, const int32_t* __restrict__ lab,
-                                 const uint8_t* __restrict__ has_void, const unsigned long long* __restrict__ best,
-                                 int32_t* __restrict__ target, int32_t* __restrict__ final_root, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    if (!vp[i] || lab[i] != i) continue;
-    int64_t t = i;
-    if (!has_void[i] && best[i] != ~0ull) {
-      const int64_t v = (int64_t)(best[i] & 0xffffffffull);
-      if (v < n && lab[v] >= 0 && lab[v] < n) t = lab[v];
+__global__ void vp_target_kernel(const int32_t* __restrict__ lab, VpScratch vp, int64_t n, int64_t n_img) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n * n_img; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t img = i / n, x = i - img * n;
+    if (lab[i] != x) continue;
+    int64_t t = x;
+    if (!vp.has_void[i] && vp.best[i] != ~0ull) {
+      const int64_t v = (int64_t)(vp.best[i] & 0xffffffffull);
+      if (v < n && lab[img * n + v] >= 0) t = lab[img * n + v];
     }
-    target[i] = (int32_t)t;
-    atomicMin(final_root + t, (int32_t)i);
+    vp.target[i] = (int32_t)t;
+    atomicMin(vp.final_root + img * n + t, (int32_t)x);
   }
 }
 
-__global__ void vp_relabel_kernel(const uint8_t* __restrict__ mask, const uint8_t* __restrict__ vp,
-                                  const int32_t* __restrict__ lab, const int32_t* __restrict__ target,
-                                  const int32_t* __restrict__ final_root, int32_t* __restrict__ out,
-                                  int32_t* __restrict__ size, uint8_t* __restrict__ has_pl, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    if (!vp[i] || lab[i] < 0 || lab[i] >= n) {
-      out[i] = -1;
-      continue;
+// Final labels (out may be null), cluster sizes and the clusters holding a
+// plastic pixel.  A thread keeps the cluster of its last pixel and adds a run
+// of the same cluster at once (a percolating cluster would otherwise take an
+// atomic on one address per warp).  grid.y: images.
+__global__ void vp_relabel_kernel(const uint8_t* __restrict__ mask, const int32_t* __restrict__ lab, VpScratch vp,
+                                  int32_t* __restrict__ out, int64_t n, int64_t n_img) {
+  for (int64_t img = blockIdx.y; img < n_img; img += gridDim.y) {
+    const int64_t b = img * n;
+    int32_t last = -1, cnt = 0;
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
+      const int32_t r = lab[b + x];
+      const int32_t f = r < 0 ? -1 : vp.final_root[b + vp.target[b + r]];
+      if (out) out[b + x] = f;
+      if (f < 0) continue;
+      if (f != last) {
+        if (cnt) atomicAdd(vp.size + b + last, cnt);
+        last = f;
+        cnt = 0;
+      }
+      cnt++;
+      if (!mask[x] && !vp.has_pl[b + f]) vp.has_pl[b + f] = 1;
     }
-    const int32_t t = target[lab[i]];
-    const int32_t f = (t >= 0 && t < n) ? final_root[t] : (int32_t)n;
-    out[i] = f < n ? f : -1;
-    if (f < n) {
-      atomicAdd(size + f, 1);
-      if (!mask[i]) has_pl[f] = 1;
-    }
+    if (cnt) atomicAdd(vp.size + b + last, cnt);
   }
 }
 
@@ -216,49 +201,51 @@ __global__ void count_kernel(const uint8_t* __restrict__ a, int64_t n, int32_t* 
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
 }
 
-__global__ void vp_stats_kernel(const int32_t* __restrict__ size, const uint8_t* __restrict__ has_pl,
-                                int32_t* __restrict__ stats, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    if (size[i] == 0) continue;
-    atomicAdd(stats, 1);
-    atomicMax(stats + 1, size[i]);
-    if (!has_pl[i]) atomicAdd(stats + 2, 1);
+// stats[4 img ..]: clusters, pixels of the largest, clusters without a plastic
+// pixel.  Final roots are roots of the first labelling.  grid.y: images.
+__global__ void vp_stats_kernel(const int32_t* __restrict__ lab, VpScratch vp, int64_t n, int64_t n_img) {
+  for (int64_t img = blockIdx.y; img < n_img; img += gridDim.y) {
+    const int64_t b = img * n;
+    int nc = 0, mx = 0, iso = 0;
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
+      if (lab[b + x] != x) continue;
+      const int32_t z = vp.size[b + x];
+      if (z == 0) continue;
+      nc++;
+      mx = max(mx, z);
+      iso += !vp.has_pl[b + x];
+    }
+    nc = __reduce_add_sync(0xffffffffu, nc);
+    iso = __reduce_add_sync(0xffffffffu, iso);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0 && nc) {
+      atomicAdd(vp.stats + 4 * img, nc);
+      atomicMax(vp.stats + 4 * img + 1, mx);
+      if (iso) atomicAdd(vp.stats + 4 * img + 2, iso);
+    }
   }
 }
 
 }  // namespace
-
-cudaError_t launch_vp_flags(const uint8_t* mask, const uint8_t* plastic, uint8_t* vp, int L, cudaStream_t s) {
-  const int64_t n = (int64_t)L * L;
-  vp_flags_kernel<<<grid_of(n), 256, 0, s>>>(mask, plastic, vp, n);
-  return cudaGetLastError();
-}
 
 cudaError_t launch_count(const uint8_t* a, int64_t n, int32_t* count_dev, cudaStream_t s) {
   count_kernel<<<grid_of(n), 256, 0, s>>>(a, n, count_dev);
   return cudaGetLastError();
 }
 
-cudaError_t launch_vp_attach(const uint8_t* mask, const uint8_t* vp, const int32_t* lab, int32_t* out, int L,
-                             void* scratch, int32_t* stats_dev, int has_voids, cudaStream_t s) {
+cudaError_t launch_vp_attach(const uint8_t* mask, const int32_t* lab, int32_t* out, int64_t n_img, int L,
+                             const VpScratch& vp, const int32_t* n_voids_dev, cudaStream_t s) {
   const int64_t n = (int64_t)L * L;
-  const int g = grid_of(n);
-  unsigned long long* best = (unsigned long long*)scratch;                  // 8 n
-  int32_t* target = (int32_t*)(best + n);                                   // 4 n
-  int32_t* final_root = target + n;                                         // 4 n
-  int32_t* size = final_root + n;                                           // 4 n
-  uint8_t* has_void = (uint8_t*)(size + n);                                 // n
-  uint8_t* has_pl = has_void + n;                                           // n
-  cudaError_t e = cudaMemsetAsync(has_void, 0, (size_t)n, s);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(stats_dev, 0, 3 * sizeof(int32_t), s);
-  if (e != cudaSuccess) return e;
-  vp_init_kernel<<<g, 256, 0, s>>>(best, final_root, size, has_pl, n);
-  vp_mark_kernel<<<g, 256, 0, s>>>(mask, lab, has_void, n);
-  if (has_voids) vp_nearest_kernel<<<g, 256, 0, s>>>(mask, vp, lab, has_void, best, L);
-  vp_target_kernel<<<g, 256, 0, s>>>(vp, lab, has_void, best, target, final_root, n);
-  vp_relabel_kernel<<<g, 256, 0, s>>>(mask, vp, lab, target, final_root, out, size, has_pl, n);
-  vp_stats_kernel<<<g, 256, 0, s>>>(size, has_pl, stats_dev, n);
+  const int g = grid_of(n * n_img);
+  const unsigned gy = (unsigned)(n_img < 32768 ? n_img : 32768);
+  // up to 16 pixels a thread in the kernels that sum per image
+  int64_t gx = (n + 4095) / 4096, most = (152 * 8 + gy - 1) / gy;
+  if (gx < most) gx = (n + 255) / 256 < most ? (n + 255) / 256 : most;
+  const dim3 per((unsigned)gx, gy);
+  vp_nearest_kernel<<<g, 256, 0, s>>>(mask, lab, vp, n_voids_dev, L, n_img);
+  vp_target_kernel<<<g, 256, 0, s>>>(lab, vp, n, n_img);
+  vp_relabel_kernel<<<per, 256, 0, s>>>(mask, lab, vp, out, n, n_img);
+  vp_stats_kernel<<<per, 256, 0, s>>>(lab, vp, n, n_img);
   return cudaGetLastError();
 }
 

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "aux_kernels.cuh"
+
 namespace epfft {
 // out(x) = in(mirror(x)) for an L x L u8 image; axes: bit 0 mirrors x1
 // (x1 -> -x1 mod L), bit 1 mirrors x2.
@@ -23,16 +25,14 @@ cudaError_t launch_plastic_flags(const T* eps, const uint8_t* mask, uint8_t* fla
 // CG2: out(x) = (in(x) + in of the four nearest neighbours) / 5, periodic.
 template <typename T>
 cudaError_t launch_avg5(const T* in, T* out, int L, cudaStream_t s);
-// Sec. 3 void-plastic clusters of one L x L image (all device buffers):
-// vp = mask | plastic, then, given lab = the clusters of vp (launch_label),
-// every cluster without a void joins the cluster of its nearest void pixel
-// (periodic Euclidean distance, ties to the smaller linear index) and
-// `out` receives the final labels (smallest linear index, -1 off the
-// phase).  stats_dev[0..2]: final clusters, pixels of the largest, clusters
-// without a plastic pixel.  scratch: 18 bytes per pixel.
-cudaError_t launch_vp_flags(const uint8_t* mask, const uint8_t* plastic, uint8_t* vp, int L, cudaStream_t s);
-cudaError_t launch_vp_attach(const uint8_t* mask, const uint8_t* vp, const int32_t* lab, int32_t* out, int L,
-                             void* scratch, int32_t* stats_dev, int has_voids, cudaStream_t s);
+// Sec. 3 void-plastic clusters of n_img L x L images (all device buffers),
+// given lab = the clusters of mask | plastic (launch_vp_label): every cluster
+// without a void joins the cluster of its nearest void pixel (periodic
+// Euclidean distance, ties to the smaller linear index); `out` (may be null)
+// receives the final labels (smallest linear index, -1 off the phase) and
+// vp.stats the counts.  n_voids_dev: void pixels of the mask.
+cudaError_t launch_vp_attach(const uint8_t* mask, const int32_t* lab, int32_t* out, int64_t n_img, int L,
+                             const VpScratch& vp, const int32_t* n_voids_dev, cudaStream_t s);
 // out(x) = [(2/3) e'_ij e'_ij]^(1/2) of a strain field (Fig. 1), e' the 3D
 // deviator of (11, 22, 33, 12), e'_12 counted twice.
 template <typename T>

@@ -33,7 +33,7 @@ def test_same_bits_as_the_passes(prec, L, tiling, monkeypatch):
             got = B.epfft_solve_batch(ctx, probs, paths, fields=True)
             # one loop launch, then mask and labels (batches of the larger sides
             # may exceed the GPU's CTAs and run the passes)
-            assert B.epfft_last_stats(ctx)["kernel_launches"] == 1 + 5 * n or (n > 1 and L >= 256)
+            assert B.epfft_last_stats(ctx)["kernel_launches"] == 1 + 4 * n or (n > 1 and L >= 256)
             monkeypatch.setenv("EPFFT_SYNC_CHECK", "1")
             ref = B.epfft_solve_batch(ctx, probs, paths, fields=True)
             monkeypatch.delenv("EPFFT_SYNC_CHECK")
