@@ -3,17 +3,10 @@
 
 namespace epfft {
 
-// Pixel x is a void iff (SplitMix64 output x of `seed`) >> 11 < thr, where the
-// i-th output of SplitMix64 is the 64-bit finaliser of seed + (i+1) gamma,
-// gamma = 0x9e3779b97f4a7c15 (Steele, Lea & Flood's generator).
 __global__ void mask_kernel(uint8_t* __restrict__ mask, int64_t n, uint64_t seed, uint64_t thr) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    uint64_t z = seed + (uint64_t)(i + 1) * 0x9e3779b97f4a7c15ull;
-    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
-    z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
-    z ^= z >> 31;
-    mask[i] = (uint8_t)((z >> 11) < thr);
+    mask[i] = void_bit(i, seed, thr);
   }
 }
 

@@ -4,6 +4,18 @@
 #include <stdint.h>
 
 namespace epfft {
+#ifdef __CUDACC__
+// Pixel i is a void iff (SplitMix64 output i of `seed`) >> 11 < thr, where the
+// i-th output of SplitMix64 is the 64-bit finaliser of seed + (i+1) gamma,
+// gamma = 0x9e3779b97f4a7c15 (Steele, Lea & Flood's generator).
+__device__ __forceinline__ uint8_t void_bit(int64_t i, uint64_t seed, uint64_t thr) {
+  uint64_t z = seed + (uint64_t)(i + 1) * 0x9e3779b97f4a7c15ull;
+  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
+  z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
+  z ^= z >> 31;
+  return (uint8_t)((z >> 11) < thr);
+}
+#endif
 cudaError_t launch_mask(uint8_t* mask, int64_t n, uint64_t seed, uint64_t thr, cudaStream_t s);
 // n_img images of L*L flags -> labels (smallest linear index of the cluster,
 // -1 off the flags) and counts_dev[n_img]; *err_dev set if a bound tripped.

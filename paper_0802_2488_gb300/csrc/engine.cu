@@ -4,6 +4,7 @@
 // labelling and copy-out.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -28,6 +29,9 @@ struct Server;
 
 // instantiation units that hold a self-check record
 constexpr int N_CHECK_UNITS = 10;
+constexpr int CTL_SOLVES = 128;  // solves of the context's device block
+constexpr int MAX_GRAPHS = 8;    // loop graphs a context keeps
+constexpr size_t STAGE_BYTES = (size_t)2 << 20;  // page-locked staging of a context
 
 struct epfft_ctx {
   int device = 0;
@@ -35,10 +39,23 @@ struct epfft_ctx {
   cudaStream_t cap = nullptr;     // stream used only to capture graph bodies
   std::vector<cudaStream_t> aux;  // fork streams of captures with parallel branches
   cudaStream_t side = nullptr;    // on-chip groups of a call that also runs a graph
-  // page-locked copies of the self-check records of the instantiation units
-  // and the records' device addresses (serving reads them on its stream)
+  // page-locked copies of the self-check records of the instantiation units,
+  // the device block a kernel gathers them in, and their device addresses
   CheckRec* h_checks = nullptr;
+  CheckRec* d_checks = nullptr;
   void* check_addr[N_CHECK_UNITS] = {};
+  // device records of the solves of a call (up to CTL_SOLVES, their refresh
+  // shadows and the control block): one block for the context's lifetime, so
+  // that the loop graphs of earlier calls, which hold its address, can be
+  // launched again
+  char* ctl_block = nullptr;
+  char* h_stage = nullptr;  // page-locked staging of a call's small transfers
+  struct LoopGraph {
+    std::tuple<int, int, int, int, int, int> key;  // L, precision, tiling, FP64 tiling, solves, general
+    cudaGraph_t graph;
+    cudaGraphExec_t exec;
+  };
+  std::deque<LoopGraph> graphs;  // latest first, at most MAX_GRAPHS
   bool own_stream = false;
   epfft_alloc_fn alloc = nullptr;
   epfft_free_fn freef = nullptr;
@@ -94,8 +111,62 @@ void dev_free(epfft_ctx* c, void* p, size_t bytes) {
 struct Arena {
   epfft_ctx* c;
   std::vector<std::pair<void*, size_t>> blocks;
+  // part of the last reserve() not handed out yet
+  char* cur = nullptr;
+  size_t left = 0;
+  // page-locked staging in use by this call, and its copies to the caller's
+  // memory once the stream is synchronised
+  size_t staged = 0;
+  struct Landing {
+    void* dst;
+    const char* src;
+    size_t bytes;
+  };
+  std::vector<Landing> landings;
+  char* stage(size_t bytes) {
+    const size_t r = round(bytes);
+    if (r > STAGE_BYTES || staged > STAGE_BYTES - r) return nullptr;
+    if (!c->h_stage && cudaMallocHost((void**)&c->h_stage, STAGE_BYTES) != cudaSuccess) {
+      c->h_stage = nullptr;
+      cudaGetLastError();
+      return nullptr;
+    }
+    char* p = c->h_stage + staged;
+    staged += r;
+    return p;
+  }
+  // Enqueues the read of device memory into host memory, in dst after the
+  // stream is synchronised and land() called.
+  cudaError_t read(void* dst, const void* dev, size_t bytes) {
+    char* p = stage(bytes);
+    if (p) landings.push_back({dst, p, bytes});
+    return cudaMemcpyAsync(p ? (void*)p : dst, dev, bytes, cudaMemcpyDeviceToHost, c->stream);
+  }
+  void land() {
+    for (const Landing& l : landings) std::memcpy(l.dst, l.src, l.bytes);
+    landings.clear();
+  }
   explicit Arena(epfft_ctx* c_) : c(c_) {}
+  static size_t round(size_t b) { return (std::max<size_t>(b, 1) + 511) & ~(size_t)511; }
+  // One block for the get()s that follow (their rounded sizes summed); an
+  // allocation through the caller's hook costs several us, and a batch takes
+  // a dozen buffers per solve.  Where the block cannot be had, get() takes
+  // each buffer from the allocator as it comes.
+  void reserve(size_t bytes) {
+    void* p = dev_alloc(c, bytes);
+    if (!p) return;
+    blocks.push_back({p, bytes});
+    cur = (char*)p;
+    left = bytes;
+  }
   void* get(size_t bytes) {
+    const size_t r = round(bytes);
+    if (r <= left) {
+      void* q = cur;
+      cur += r;
+      left -= r;
+      return q;
+    }
     void* p = dev_alloc(c, bytes);
     if (p) blocks.push_back({p, bytes});
     return p;
@@ -190,9 +261,18 @@ cudaError_t read_check_all(CheckRec* out) {
   return cudaSuccess;
 }
 
-// Enqueues on stream s the copies of every unit's self-check record into the
-// context's page-locked buffer (read them once s is synchronised); the
-// buffer and the records' addresses are set up on first use.
+struct CheckAddrs {
+  const CheckRec* p[N_CHECK_UNITS];
+};
+__global__ void gather_checks_kernel(CheckAddrs a, CheckRec* out) {
+  const int i = threadIdx.x;
+  if (i < N_CHECK_UNITS) out[i] = a.p[i] ? *a.p[i] : CheckRec{};
+}
+
+// Enqueues on stream s the read of every unit's self-check record into the
+// context's page-locked buffer (read it once s is synchronised): one kernel
+// gathers them, one copy brings them.  The buffers and the records' addresses
+// are set up on first use.
 cudaError_t enqueue_check_reads(epfft_ctx* c, cudaStream_t s) {
   if (!c->h_checks) {
     cudaError_t e;
@@ -207,20 +287,41 @@ cudaError_t enqueue_check_reads(epfft_ctx* c, cudaStream_t s) {
     if ((e = check_record_onchip(&a[7])) != cudaSuccess) return e;
     if ((e = check_record_resident<float>(&a[8])) != cudaSuccess) return e;
     if ((e = check_record_resident<double>(&a[9])) != cudaSuccess) return e;
+    CheckRec* d = (CheckRec*)dev_alloc(c, sizeof(CheckRec) * N_CHECK_UNITS);
+    if (!d) return cudaErrorMemoryAllocation;
     CheckRec* h = nullptr;
-    if ((e = cudaMallocHost((void**)&h, sizeof(CheckRec) * N_CHECK_UNITS)) != cudaSuccess) return e;
+    if ((e = cudaMallocHost((void**)&h, sizeof(CheckRec) * N_CHECK_UNITS)) != cudaSuccess) {
+      dev_free(c, d, sizeof(CheckRec) * N_CHECK_UNITS);
+      return e;
+    }
     for (int i = 0; i < N_CHECK_UNITS; i++) {
       c->check_addr[i] = a[i];
       h[i] = CheckRec{};
     }
+    c->d_checks = d;
     c->h_checks = h;
   }
+  CheckAddrs ca;
+  for (int i = 0; i < N_CHECK_UNITS; i++) ca.p[i] = (const CheckRec*)c->check_addr[i];
+  gather_checks_kernel<<<1, 32, 0, s>>>(ca, c->d_checks);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return cudaMemcpyAsync(c->h_checks, c->d_checks, sizeof(CheckRec) * N_CHECK_UNITS, cudaMemcpyDeviceToHost, s);
+}
+
+// After the stream of enqueue_check_reads was synchronised: EPFFT_ERR_CUDA (with
+// a message, the records cleared) if a check fired.
+int check_result(epfft_ctx* c) {
   for (int i = 0; i < N_CHECK_UNITS; i++) {
-    if (!c->check_addr[i]) continue;
-    cudaError_t e = cudaMemcpyAsync(&c->h_checks[i], c->check_addr[i], sizeof(CheckRec), cudaMemcpyDeviceToHost, s);
-    if (e != cudaSuccess) return e;
+    const CheckRec cr = c->h_checks[i];
+    if (!cr.code) continue;
+    CheckRec clr;
+    if (read_check_all(&clr) != cudaSuccess) cudaGetLastError();
+    fprintf(stderr, "epfft: device self-check %d failed (index %lld, bound %lld, at %d)\n", cr.code,
+            (long long)cr.index, (long long)cr.bound, cr.where);
+    return EPFFT_ERR_CUDA;
   }
-  return cudaSuccess;
+  return EPFFT_OK;
 }
 
 // Raises the shared-memory limits of the kernels of one tiling (once).
@@ -335,6 +436,13 @@ struct Batch {
   Solve* d_shadow = nullptr;
   std::vector<Solve> h_shadow;  // serving: host copy of the shadow slots
   bool resident = false;  // ran on the resident schedule
+  bool own_ctl = false;   // d_solves, d_shadow and d_ctl are in the context's block
+  // of setup_batch: host copy of an upload too large for the staging, the
+  // records and the flags of all increments, solve by solve
+  std::vector<char> h_up;
+  Record* d_rec = nullptr;
+  uint8_t* flags = nullptr;
+  size_t tot_inc = 0;
   int64_t refreshes = 0;  // refreshes launched from the host (fixed-step loops)
   std::vector<Solve> h_solves;
   std::vector<int32_t> n_inc;
@@ -393,12 +501,22 @@ size_t solve_footprint(int L, int prec, int row_ctas, int n_inc) {
          r(sizeof(double) * 4 * (size_t)n_inc) + r(sizeof(Record) * (size_t)n_inc);
 }
 
-// Allocates (through `get`) and initialises the device state of one solve on
-// stream s: buffers, path, mask, starting strain (eps0: device pointer or
-// null for an unstrained lattice).  Fills the host record S.
+// Buffers of a solve that are part of a batch's (null: taken from `get`).
+struct BatchPart {
+  uint8_t* flags = nullptr;
+  double* path = nullptr;
+  Record* rec = nullptr;
+};
+
+// Allocates (through `get`) the device state of one solve and fills its host
+// record S.  Enqueued on stream s: the copies of a caller's mask and starting
+// strain (eps0: device pointer, or null for an unstrained lattice).  In a
+// batch (bp) the path, the cleared records, a generated mask and the zeros
+// of the rest come from the batch's upload and batch_init_kernel; else they
+// are enqueued here.
 template <typename Get>
 int init_solve(Get&& get, const PassShape& sh, int L, int prec, const epfft_problem& p, const double* path,
-               int n_inc, const void* eps0, cudaStream_t s, Solve& S) {
+               int n_inc, const void* eps0, cudaStream_t s, Solve& S, const BatchPart* bp = nullptr) {
   const size_t LL = (size_t)L * L, rs = real_size(prec);
   std::memset(&S, 0, sizeof(S));
   S.lam = p.lambda;
@@ -423,9 +541,9 @@ int init_solve(Get&& get, const PassShape& sh, int L, int prec, const epfft_prob
   void* spec = get(3 * LL * spec_real_size(prec));
   double* part = (double*)get(sizeof(double) * PART_STRIDE * (size_t)sh.row_ctas);
   uint8_t* mask = (uint8_t*)get(LL);
-  uint8_t* flags = (uint8_t*)get(LL * (size_t)n_inc);
-  double* dpath = (double*)get(sizeof(double) * 4 * (size_t)n_inc);
-  Record* rec = (Record*)get(sizeof(Record) * (size_t)n_inc);
+  uint8_t* flags = bp ? bp->flags : (uint8_t*)get(LL * (size_t)n_inc);
+  double* dpath = bp ? bp->path : (double*)get(sizeof(double) * 4 * (size_t)n_inc);
+  Record* rec = bp ? bp->rec : (Record*)get(sizeof(Record) * (size_t)n_inc);
   if (!eps0d || !eps1d || !sig0d || !sig1d || !spec || !part || !mask || !flags || !dpath || !rec)
     return EPFFT_ERR_OOM;
   S.eps[0] = eps0d;
@@ -446,8 +564,10 @@ int init_solve(Get&& get, const PassShape& sh, int L, int prec, const epfft_prob
       S.deps[k] = get(4 * LL * 4);
       S.dsig[k] = get(4 * LL * 4);
       if (!S.deps[k] || !S.dsig[k]) return EPFFT_ERR_OOM;
-      CK(cudaMemsetAsync(S.deps[k], 0, 4 * LL * 4, s));
-      CK(cudaMemsetAsync(S.dsig[k], 0, 4 * LL * 4, s));
+      if (!bp) {
+        CK(cudaMemsetAsync(S.deps[k], 0, 4 * LL * 4, s));
+        CK(cudaMemsetAsync(S.dsig[k], 0, 4 * LL * 4, s));
+      }
     }
     S.base[0] = get(4 * LL * 4);
     S.base[1] = get(4 * LL * 4);
@@ -458,29 +578,73 @@ int init_solve(Get&& get, const PassShape& sh, int L, int prec, const epfft_prob
     if (!S.base[0] || !S.base[1] || !S.base[2] || !S.spec64 || !S.refpart) return EPFFT_ERR_OOM;
     S.zero_mean = 1;
   }
-  CK(cudaMemcpyAsync(dpath, path, sizeof(double) * 4 * (size_t)n_inc, cudaMemcpyHostToDevice, s));
-  CK(cudaMemsetAsync(rec, 0, sizeof(Record) * (size_t)n_inc, s));
+  if (!bp) {
+    CK(cudaMemcpyAsync(dpath, path, sizeof(double) * 4 * (size_t)n_inc, cudaMemcpyHostToDevice, s));
+    CK(cudaMemsetAsync(rec, 0, sizeof(Record) * (size_t)n_inc, s));
+  }
   if (p.mask) {
     CK(cudaMemcpyAsync(mask, p.mask, LL, p.mask_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-  } else {
+  } else if (!bp) {
     CK(launch_mask(mask, (int64_t)LL, p.seed, void_threshold(p.void_fraction), s));
   }
   if (eps0) {
     CK(cudaMemcpyAsync(eps0d, eps0, 4 * LL * rs, cudaMemcpyDeviceToDevice, s));
     for (int k = 0; k < 4; k++) S.Eprev[k] = path[k];
-  } else {
+  } else if (!bp) {
     CK(cudaMemsetAsync(eps0d, 0, 4 * LL * rs, s));
   }
   return EPFFT_OK;
 }
+
+// What batch_init_kernel does for a solve: generate its mask, clear its
+// starting strain.
+struct InitItem {
+  uint64_t seed, thr;
+  int32_t gen, zero;
+};
+// Starting state of a batch: generated masks, zero strains and (defect form)
+// zero differences, four pixels a thread; grid.y: solves.
+__global__ void __launch_bounds__(256) batch_init_kernel(const Solve* __restrict__ solves,
+                                                         const InitItem* __restrict__ items, int64_t LL, int rs,
+                                                         int dc) {
+  const Solve& S = solves[blockIdx.y];
+  const InitItem it = items[blockIdx.y];
+  uint8_t* mask = const_cast<uint8_t*>(S.mask);
+  const int4 z = make_int4(0, 0, 0, 0);
+  for (int64_t i = 4 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x); i < LL; i += 4 * (int64_t)gridDim.x * blockDim.x) {
+    if (it.gen) {
+      uchar4 m;
+      m.x = void_bit(i, it.seed, it.thr);
+      m.y = void_bit(i + 1, it.seed, it.thr);
+      m.z = void_bit(i + 2, it.seed, it.thr);
+      m.w = void_bit(i + 3, it.seed, it.thr);
+      *reinterpret_cast<uchar4*>(mask + i) = m;
+    }
+    if (it.zero) {
+      int4* e = reinterpret_cast<int4*>(S.eps[0]) + i * (rs / 4);
+      for (int k = 0; k < rs; k++) e[k] = z;
+    }
+    if (dc)
+      for (int k = 0; k < 4; k++) {
+        reinterpret_cast<int4*>(S.deps[0])[i + k] = z;
+        reinterpret_cast<int4*>(S.deps[1])[i + k] = z;
+        reinterpret_cast<int4*>(S.dsig[0])[i + k] = z;
+        reinterpret_cast<int4*>(S.dsig[1])[i + k] = z;
+      }
+  }
+}
+
+size_t ctl_block_bytes() { return Arena::round(sizeof(Solve) * CTL_SOLVES) * 2 + Arena::round(sizeof(BatchCtl)); }
 
 // Builds the device state of n problems.  eps0 (optional, device) gives the
 // starting local strain of every solve (then the first increment starts
 // from it unshifted); otherwise the lattice starts unstrained.
 // onchip: the on-chip schedule may be used (the device-driven solves; the
 // fixed-step loops run the two passes).
+// own_ctl: the solves' records may live in the context's block (one batch of a
+// call), so that its loop graph can be kept.
 int setup_batch(epfft_ctx* c, Arena& A, Batch& B, int n, const epfft_problem* probs,
-                const epfft_path* paths, const void* const* eps0, bool onchip = true) {
+                const epfft_path* paths, const void* const* eps0, bool onchip = true, bool own_ctl = false) {
   B.L = probs[0].L;
   B.prec = probs[0].precision;
   B.nb = n;
@@ -501,42 +665,107 @@ int setup_batch(epfft_ctx* c, Arena& A, Batch& B, int n, const epfft_problem* pr
   if (rc) return rc;
   B.h_solves.resize(n);
   B.n_inc.resize(n);
+  // one device block for the batch: per solve its buffers, then the flags of
+  // every increment, and the upload (paths, solves, shadows, control block,
+  // start items) followed by the records, which come back in one copy
+  const size_t LL = (size_t)B.L * B.L;
+  const bool dc = B.prec == EPFFT_FP32_DEFECT;
+  size_t tot_inc = 0, bytes = 0;
+  for (int i = 0; i < n; i++) {
+    tot_inc += (size_t)paths[i].n_inc;
+    bytes += solve_footprint(B.L, B.prec, B.sh.row_ctas, 0);
+  }
+  // the context's own records where they fit and no earlier batch of this
+  // call has them
+  const bool own = own_ctl && n <= CTL_SOLVES;
+  if (own && !c->ctl_block) c->ctl_block = (char*)dev_alloc(c, ctl_block_bytes());
+  const bool ctl = own && c->ctl_block;
+  auto R = [](size_t b) { return Arena::round(b); };
+  const size_t o_path = 0, o_item = o_path + R(sizeof(double) * 4 * tot_inc),
+               o_solve = o_item + R(sizeof(InitItem) * (size_t)n), o_shadow = o_solve + R(sizeof(Solve) * (size_t)n),
+               o_ctl = o_shadow + R(dc ? sizeof(Solve) * (size_t)n : 0), up_bytes = o_ctl + R(sizeof(BatchCtl));
+  const size_t rec_bytes = sizeof(Record) * tot_inc;
+  A.reserve(bytes + R(LL * tot_inc) + up_bytes + R(rec_bytes));
+  uint8_t* flags = (uint8_t*)A.get(LL * tot_inc);
+  char* up = (char*)A.get(up_bytes);
+  B.d_rec = (Record*)A.get(rec_bytes);
+  if (!flags || !up || !B.d_rec) return EPFFT_ERR_OOM;
+  B.flags = flags;
+  B.tot_inc = tot_inc;
+  char* h = A.stage(up_bytes);
+  if (!h) {
+    B.h_up.resize(up_bytes);
+    h = B.h_up.data();
+  }
+  std::memset(h, 0, up_bytes);
+  InitItem* items = (InitItem*)(h + o_item);
   int64_t max_body = 0;
+  size_t off = 0;
+  bool init = dc;
   for (int i = 0; i < n; i++) {
     const epfft_problem& p = probs[i];
+    const size_t ni = (size_t)paths[i].n_inc;
     B.n_inc[i] = paths[i].n_inc;
-    rc = init_solve([&](size_t b) { return A.get(b); }, B.sh, B.L, B.prec, p, paths[i].E, paths[i].n_inc,
-                    eps0 ? eps0[i] : nullptr, c->stream, B.h_solves[i]);
+    std::memcpy(h + o_path + sizeof(double) * 4 * off, paths[i].E, sizeof(double) * 4 * ni);
+    BatchPart part;
+    part.flags = flags + LL * off;
+    part.path = (double*)(up + o_path) + 4 * off;
+    part.rec = B.d_rec + off;
+    off += ni;
+    const void* e0 = eps0 ? eps0[i] : nullptr;
+    rc = init_solve([&](size_t b) { return A.get(b); }, B.sh, B.L, B.prec, p, paths[i].E, paths[i].n_inc, e0,
+                    c->stream, B.h_solves[i], &part);
     if (rc) return rc;
+    items[i] = InitItem{p.seed, void_threshold(p.void_fraction), p.mask ? 0 : 1, e0 ? 0 : 1};
+    init |= items[i].gen || items[i].zero;
     B.h_solves[i].ref_every = c->defect_refresh;
     const int64_t need = (int64_t)paths[i].n_inc * ((int64_t)p.max_iter + 2) + 1;
     if (need > max_body) max_body = need;
   }
-  B.d_solves = (Solve*)A.get(sizeof(Solve) * (size_t)n);
-  B.d_ctl = (BatchCtl*)A.get(sizeof(BatchCtl));
-  if (!B.d_solves || !B.d_ctl) return EPFFT_ERR_OOM;
-  CK(cudaMemcpyAsync(B.d_solves, B.h_solves.data(), sizeof(Solve) * (size_t)n, cudaMemcpyHostToDevice, c->stream));
-  if (B.prec == EPFFT_FP32_DEFECT) {
-    // shadow solves of the refresh's FP64 column pass: the FP64 spectrum
-    // and 0 at q = 0 (ref_forward mirrors phase, increment and buffer)
-    std::vector<Solve> sh = B.h_solves;
-    for (auto& z : sh) {
+  std::memcpy(h + o_solve, B.h_solves.data(), sizeof(Solve) * (size_t)n);
+  if (dc)
+    for (int i = 0; i < n; i++) {
+      // shadow solves of the refresh's FP64 column pass: the FP64 spectrum
+      // and 0 at q = 0 (ref_forward mirrors phase, increment and buffer)
+      Solve z = B.h_solves[i];
       z.spec = z.spec64;
       z.zero_mean = 1;
+      std::memcpy(h + o_shadow + sizeof(Solve) * (size_t)i, &z, sizeof(z));
     }
-    B.d_shadow = (Solve*)A.get(sizeof(Solve) * (size_t)n);
-    if (!B.d_shadow) return EPFFT_ERR_OOM;
-    CK(cudaMemcpyAsync(B.d_shadow, sh.data(), sizeof(Solve) * (size_t)n, cudaMemcpyHostToDevice, c->stream));
-    // the host copy leaves this scope: wait for the upload
-    CK(cudaStreamSynchronize(c->stream));
-  }
   BatchCtl bc;
   std::memset(&bc, 0, sizeof(bc));
   bc.active = n;
   bc.max_body_iters = max_body + 8;
-  bc.dc = B.prec == EPFFT_FP32_DEFECT;
+  bc.dc = dc;
   B.max_body = bc.max_body_iters;
-  CK(cudaMemcpyAsync(B.d_ctl, &bc, sizeof(bc), cudaMemcpyHostToDevice, c->stream));
+  std::memcpy(h + o_ctl, &bc, sizeof(bc));
+  CK(cudaMemcpyAsync(up, h, up_bytes, cudaMemcpyHostToDevice, c->stream));
+  CK(cudaMemsetAsync(B.d_rec, 0, rec_bytes, c->stream));
+  B.d_solves = (Solve*)(up + o_solve);
+  B.d_shadow = dc ? (Solve*)(up + o_shadow) : nullptr;
+  B.d_ctl = (BatchCtl*)(up + o_ctl);
+  if (init) {
+    const int64_t q = ((int64_t)LL / 4 + 255) / 256, most = std::max<int64_t>(1, 152 * 16 / n);
+    // grid.y holds at most 65535 solves
+    for (int i0 = 0; i0 < n; i0 += 65535) {
+      batch_init_kernel<<<dim3((unsigned)std::min(q, most), (unsigned)std::min(n - i0, 65535)), 256, 0, c->stream>>>(
+          B.d_solves + i0, (const InitItem*)(up + o_item) + i0, (int64_t)LL, (int)real_size(B.prec), dc ? 1 : 0);
+      if (cudaGetLastError() != cudaSuccess) return EPFFT_ERR_CUDA;
+    }
+  }
+  if (ctl) {
+    Solve* own_solves = (Solve*)c->ctl_block;
+    Solve* own_shadow = (Solve*)(c->ctl_block + R(sizeof(Solve) * CTL_SOLVES));
+    BatchCtl* own_bc = (BatchCtl*)(c->ctl_block + 2 * R(sizeof(Solve) * CTL_SOLVES));
+    CK(cudaMemcpyAsync(own_solves, B.d_solves, sizeof(Solve) * (size_t)n, cudaMemcpyDeviceToDevice, c->stream));
+    if (dc)
+      CK(cudaMemcpyAsync(own_shadow, B.d_shadow, sizeof(Solve) * (size_t)n, cudaMemcpyDeviceToDevice, c->stream));
+    CK(cudaMemcpyAsync(own_bc, B.d_ctl, sizeof(BatchCtl), cudaMemcpyDeviceToDevice, c->stream));
+    B.d_solves = own_solves;
+    if (dc) B.d_shadow = own_shadow;
+    B.d_ctl = own_bc;
+    B.own_ctl = true;
+  }
   return EPFFT_OK;
 }
 
@@ -690,8 +919,36 @@ int enqueue_resident(epfft_ctx* c, Arena& A, Batch& B, int g) {
   return EPFFT_OK;
 }
 
-// Runs the device-side loop of a batch to completion (one graph launch).
+// Runs the device-side loop of a batch to completion (one graph launch).  A
+// graph over the context's own records is kept for later calls of the same
+// shape (building one costs some 200 us); the latest MAX_GRAPHS are.
 int run_graph(epfft_ctx* c, Batch& B) {
+  const auto key = std::make_tuple(B.L, B.prec, B.var, B.var64, B.nb, B.general);
+  if (B.own_ctl) {
+    auto it = c->graphs.begin();
+    while (it != c->graphs.end() && it->key != key) ++it;
+    if (it == c->graphs.end()) {
+      epfft_ctx::LoopGraph g{key, nullptr, nullptr};
+      int rc = build_loop_graph(c, B, &g.graph, &g.exec);
+      if (rc) return rc;
+      if ((int)c->graphs.size() >= MAX_GRAPHS) {
+        // its last launch ended with the call that made it
+        cudaGraphExecDestroy(c->graphs.back().exec);
+        cudaGraphDestroy(c->graphs.back().graph);
+        c->graphs.pop_back();
+      }
+      c->graphs.push_front(g);
+    } else if (it != c->graphs.begin()) {
+      const epfft_ctx::LoopGraph g = *it;
+      c->graphs.erase(it);
+      c->graphs.push_front(g);
+    }
+    if (cudaGraphLaunch(c->graphs.front().exec, c->stream) != cudaSuccess) {
+      cudaGetLastError();
+      return EPFFT_ERR_CUDA;
+    }
+    return EPFFT_OK;
+  }
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   int rc = build_loop_graph(c, B, &graph, &exec);
@@ -852,7 +1109,6 @@ int run_host_loop(epfft_ctx* c, Batch& B, int64_t steps) {
       B.refreshes += 1;
     }
   }
-  CK(cudaStreamSynchronize(c->stream));
   return EPFFT_OK;
 }
 
@@ -904,6 +1160,36 @@ int run_checked(epfft_ctx* c, Batch& B) {
       return EPFFT_OK;
     }
   }
+}
+
+// Copies the accepted strain of a finished solve to `out` (words of 16 bytes).
+__global__ void __launch_bounds__(256) accepted_strain_kernel(const Solve* S, const BatchCtl* bc, int4* __restrict__ out,
+                                                              int64_t words) {
+  if (S->phase != PH_DONE || bc->timed_out) return;
+  const int4* in = reinterpret_cast<const int4*>(S->eps[S->cur]);
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < words; i += (int64_t)gridDim.x * blockDim.x)
+    out[i] = in[i];
+}
+
+// Enqueues the cluster counts of every increment of a batch (flags of all
+// solves in a row) and their copy into `counts`, followed by the labelling's
+// error flag; up to 256 MB of label scratch at a time.
+int count_clusters(epfft_ctx* c, Arena& A, Batch& B, std::vector<int32_t>& counts, int* launches) {
+  const size_t LL = (size_t)B.L * B.L;
+  size_t step = std::max<size_t>(1, std::min(B.tot_inc, ((size_t)256 << 20) / (sizeof(int32_t) * LL)));
+  int32_t* lab = (int32_t*)A.get(sizeof(int32_t) * LL * step);
+  if (!lab && step > 1) lab = (int32_t*)A.get(sizeof(int32_t) * LL * (step = 1));
+  int32_t* dc = (int32_t*)A.get(sizeof(int32_t) * (B.tot_inc + 1));
+  if (!lab || !dc) return EPFFT_ERR_OOM;
+  CK(cudaMemsetAsync(dc + B.tot_inc, 0, sizeof(int32_t), c->stream));
+  for (size_t k = 0; k < B.tot_inc; k += step) {
+    const size_t m = std::min(step, B.tot_inc - k);
+    CK(launch_label(B.flags + LL * k, lab, (int64_t)m, B.L, 1, dc + k, dc + B.tot_inc, c->stream, false));
+    *launches += 3;
+  }
+  counts.assign(B.tot_inc + 1, 0);
+  CK(A.read(counts.data(), dc, sizeof(int32_t) * (B.tot_inc + 1)));
+  return EPFFT_OK;
 }
 
 // Labels the per-increment plastic flags of every solve and fills
@@ -1032,7 +1318,7 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
     }
     const char* chk0 = getenv("EPFFT_SYNC_CHECK");
     const bool onchip = host_steps == 0 && !(chk0 && chk0[0] == '1');
-    int rc = setup_batch(c, A, Bs[g], (int)pg.size(), pg.data(), qg.data(), eps0, onchip);
+    int rc = setup_batch(c, A, Bs[g], (int)pg.size(), pg.data(), qg.data(), eps0, onchip, G == 1);
     if (rc) return rc;
     Bp[g] = &Bs[g];
   }
@@ -1042,7 +1328,6 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
     for (int g = 0; g < G && !rc; g++) rc = run_checked(c, Bs[g]);
   } else if (const int g = G == 1 ? resident_ctas(c, Bs[0].L, Bs[0].prec, Bs[0].var, Bs[0].nb, Bs[0].sh.row_ctas) : 0) {
     rc = enqueue_resident(c, A, Bs[0], g);
-    if (!rc && cudaStreamSynchronize(c->stream) != cudaSuccess) rc = EPFFT_ERR_CUDA;
   } else if (host_steps > 0) {
     rc = run_host_loop(c, Bs[0], host_steps);
   } else {
@@ -1069,34 +1354,50 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
     else if (!rc && stream_groups.size() > 1) rc = run_mixed_graph(c, A, stream_groups);
     // the side stream's work ends before anything is read back or freed
     if (ocs != c->stream && cudaStreamSynchronize(ocs) != cudaSuccess && !rc) rc = EPFFT_ERR_CUDA;
-    if (!rc && cudaStreamSynchronize(c->stream) != cudaSuccess) rc = EPFFT_ERR_CUDA;
   }
   if (rc) return rc;
-  // read back the solve states, the control blocks and the records
+  // behind the loop on the same stream: the accepted strain of a solve whose
+  // caller wants it in place, and, when no fields are asked for, the cluster
+  // counts; then one read-back of the solve states, the control blocks, the
+  // records, the counts and the self-check records
+  int launches = 1;  // the gathering of the self-check records
+  if (eps_out)
+    for (int i = 0; i < n; i++)
+      if (eps_out[i]) {
+        Batch& B = Bs[where[i]];
+        const int64_t words = (int64_t)B.L * B.L * (int64_t)real_size(B.prec) / 4;
+        accepted_strain_kernel<<<(unsigned)std::min<int64_t>((words + 255) / 256, 152 * 16), 256, 0, c->stream>>>(
+            B.d_solves + slot[i], B.d_ctl, (int4*)eps_out[i], words);
+        if (cudaGetLastError() != cudaSuccess) return EPFFT_ERR_CUDA;
+        launches++;
+      }
+  std::vector<std::vector<int32_t>> counts(G);  // clusters per increment, then the labelling's error flag
+  if (!fields)
+    for (int g = 0; g < G; g++) {
+      rc = count_clusters(c, A, Bs[g], counts[g], &launches);
+      if (rc) return rc;
+    }
   std::vector<BatchCtl> bc(G);
+  std::vector<std::vector<Record>> rec(G);
   for (int g = 0; g < G; g++) {
-    CK(cudaMemcpyAsync(Bs[g].h_solves.data(), Bs[g].d_solves, sizeof(Solve) * (size_t)Bs[g].nb,
-                       cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaMemcpyAsync(&bc[g], Bs[g].d_ctl, sizeof(BatchCtl), cudaMemcpyDeviceToHost, c->stream));
+    rec[g].resize(Bs[g].tot_inc);
+    CK(A.read(Bs[g].h_solves.data(), Bs[g].d_solves, sizeof(Solve) * (size_t)Bs[g].nb));
+    CK(A.read(&bc[g], Bs[g].d_ctl, sizeof(BatchCtl)));
+    CK(A.read(rec[g].data(), Bs[g].d_rec, sizeof(Record) * Bs[g].tot_inc));
   }
+  CK(enqueue_check_reads(c, c->stream));
   CK(cudaStreamSynchronize(c->stream));
+  A.land();
+  rc = check_result(c);
+  if (rc) return rc;
   std::vector<std::vector<std::vector<Record>>> recs(G);
   for (int g = 0; g < G; g++) {
-    recs[g].resize(Bs[g].nb);
+    size_t off = 0;
     for (int j = 0; j < Bs[g].nb; j++) {
-      recs[g][j].resize(Bs[g].n_inc[j]);
-      CK(cudaMemcpyAsync(recs[g][j].data(), Bs[g].h_solves[j].rec, sizeof(Record) * (size_t)Bs[g].n_inc[j],
-                         cudaMemcpyDeviceToHost, c->stream));
-    }
-  }
-  CK(cudaStreamSynchronize(c->stream));
-  {
-    CheckRec cr;
-    CK(read_check_all(&cr));
-    if (cr.code) {
-      fprintf(stderr, "epfft: device self-check %d failed (index %lld, bound %lld, at %d)\n", cr.code,
-              (long long)cr.index, (long long)cr.bound, cr.where);
-      return EPFFT_ERR_CUDA;
+      recs[g].emplace_back(rec[g].begin() + off, rec[g].begin() + off + Bs[g].n_inc[j]);
+      if (!fields)
+        for (int k = 0; k < Bs[g].n_inc[j]; k++) recs[g][j][k].n_clusters = counts[g][off + k];
+      off += (size_t)Bs[g].n_inc[j];
     }
   }
   {
@@ -1118,14 +1419,15 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
     if (streaming > 1) k += steps;  // the loop-condition kernel of the mixed graph
     // the defect form's refreshes: from the host, and the loop body's node
     for (int g = 0; g < G; g++) k += 4 * (Bs[g].refreshes + bc[g].refresh_runs);
-    // per solve the mask kernel (when generated) and the three labelling kernels
-    for (int i = 0; i < n; i++) k += (probs[i].mask ? 0 : 1) + 3;
+    // the starting state of every batch, the kernels behind the loop, and with
+    // fields the three labelling kernels of every solve
+    k += G + launches + (fields ? 3 * (int64_t)n : 0);
     c->last.loop_steps = steps;
     c->last.kernel_launches = k;
     c->last.iterations = its;
   }
   for (int g = 0; g < G; g++)
-    if (bc[g].timed_out) return EPFFT_ERR_DEVICE_TIMEOUT;
+    if (bc[g].timed_out || (!fields && counts[g].back())) return EPFFT_ERR_DEVICE_TIMEOUT;
   // The fields go out on a copy stream while the work stream labels: first
   // the final strains and the plastic flags, then each solve's labels as
   // soon as they are written.  The copy stream's work ends before the call
@@ -1150,17 +1452,16 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
       rc = copy_out(B, B.h_solves[slot[i]], slot[i], &fields[i], cs);
       if (rc) return rc;
     }
-  for (int g = 0; g < G; g++) {
+  for (int g = 0; fields && g < G; g++) {
     // the caller's label buffers of the batch's solves (labels are copied
     // out by the labelling itself; copy_out does the other fields)
     std::vector<int32_t*> lab_out(Bs[g].nb, nullptr);
     std::vector<cudaMemcpyKind> kind(Bs[g].nb, cudaMemcpyDeviceToHost);
-    if (fields)
-      for (int j = 0; j < Bs[g].nb; j++) {
-        const epfft_fields& f = fields[members[g][j]];
-        lab_out[j] = (int32_t*)f.labels;
-        kind[j] = f.on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-      }
+    for (int j = 0; j < Bs[g].nb; j++) {
+      const epfft_fields& f = fields[members[g][j]];
+      lab_out[j] = (int32_t*)f.labels;
+      kind[j] = f.on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+    }
     rc = label_batch(c, A, Bs[g], recs[g], lab_out, kind, cs);
     if (rc) return rc;
   }
@@ -1172,16 +1473,13 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
     const Solve& S = B.h_solves[j];
     if (S.phase != PH_DONE && S.status == 0) return EPFFT_ERR_DEVICE_TIMEOUT;
     if (records) std::memcpy(records[i], R.data(), sizeof(Record) * (size_t)B.n_inc[j]);
-    if (eps_out && eps_out[i])
-      CK(cudaMemcpyAsync(eps_out[i], S.eps[S.cur], 4 * (size_t)B.L * B.L * real_size(B.prec),
-                         cudaMemcpyDeviceToDevice, c->stream));
     if (iter_rec) std::memcpy(&iter_rec[i], &R[B.n_inc[j] - 1], sizeof(Record));
     for (int k = 0; k < B.n_inc[j]; k++) {
       if (R[k].status == 2) status = EPFFT_ERR_NUMERIC;
       else if (R[k].status == 1 && status == EPFFT_OK) status = EPFFT_NOT_CONVERGED;
     }
   }
-  CK(cudaStreamSynchronize(c->stream));
+  if (fields) CK(cudaStreamSynchronize(c->stream));
   if (cs != c->stream) CK(cudaStreamSynchronize(cs));
   return status;
 }
@@ -1497,8 +1795,20 @@ int serve_admit(epfft_ctx* c, Server& S) {
     p.mask_on_device = 0;
     if (!p.mask) c->last.kernel_launches += 1;  // the mask kernel
     Solve hs;
+    // one block for the request's buffers (t.bytes is the sum of their rounded
+    // sizes); one by one where it cannot be had
+    char* blk = (char*)dev_alloc(c, t.bytes);
+    size_t left = blk ? t.bytes : 0;
+    if (blk) sl.blocks.push_back({blk, t.bytes});
     rc = init_solve(
         [&](size_t b) {
+          const size_t r = Arena::round(b);
+          if (r <= left) {
+            void* q = blk;
+            blk += r;
+            left -= r;
+            return q;
+          }
           void* q = dev_alloc(c, b);
           if (q) sl.blocks.push_back({q, b});
           return q;
@@ -1655,7 +1965,14 @@ void epfft_destroy(epfft_ctx* c) {
   cudaSetDevice(c->device);
   if (c->server) epfft_serve_close(c);
   cudaStreamSynchronize(c->stream);
+  for (auto& g : c->graphs) {
+    cudaGraphExecDestroy(g.exec);
+    cudaGraphDestroy(g.graph);
+  }
   for (auto& t : c->tables) dev_free(c, t.second.dev, t.second.bytes);
+  if (c->h_stage) cudaFreeHost(c->h_stage);
+  if (c->ctl_block) dev_free(c, c->ctl_block, ctl_block_bytes());
+  if (c->d_checks) dev_free(c, c->d_checks, sizeof(CheckRec) * N_CHECK_UNITS);
   cudaStreamSynchronize(c->stream);
   cudaStreamDestroy(c->cap);
   for (cudaStream_t a : c->aux) cudaStreamDestroy(a);
@@ -2175,19 +2492,25 @@ int epfft_project(epfft_ctx* ctx, int32_t L, int32_t precision, double lambda0, 
   if (!rc) rc = ensure_prepared(ctx, L, precision, var);
   if (rc) return rc;
   const size_t LL = (size_t)L * L, rs = real_size(precision);
+  struct {
+    Solve S;
+    double E[4];
+  } up;
+  A.reserve(Arena::round(3 * LL * rs) + Arena::round(sizeof(up)));
   void* spec = A.get(3 * LL * rs);
-  double* dpath = (double*)A.get(4 * sizeof(double));
-  Solve* ds = (Solve*)A.get(sizeof(Solve));
-  if (!spec || !dpath || !ds) return EPFFT_ERR_OOM;
-  Solve S;
-  std::memset(&S, 0, sizeof(S));
+  char* dev = (char*)A.get(sizeof(up));
+  if (!spec || !dev) return EPFFT_ERR_OOM;
+  Solve* ds = (Solve*)dev;
+  double* dpath = (double*)(dev + offsetof(decltype(up), E));
+  std::memset(&up, 0, sizeof(up));
+  std::memcpy(up.E, E, sizeof(up.E));
+  Solve& S = up.S;
   S.lam0 = lambda0;
   S.mu0 = mu0;
   S.path = dpath;
   S.spec = spec;
   S.phase = PH_ITER;
-  CK(cudaMemcpyAsync(dpath, E, 4 * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
-  CK(cudaMemcpyAsync(ds, &S, sizeof(S), cudaMemcpyHostToDevice, ctx->stream));
+  CK(cudaMemcpyAsync(dev, &up, sizeof(up), cudaMemcpyHostToDevice, ctx->stream));
   if (precision == EPFFT_FP32) {
     CK(launch_row_forward<float>(L, var, ctx->stream, p_dev, spec, tw));
     CK(launch_col<float>(L, var, 1, ctx->stream, ds, tw, ktab, 0, 0));
@@ -2213,6 +2536,7 @@ int epfft_displacement(epfft_ctx* ctx, int32_t L, int32_t precision, const void*
   if (!rc) rc = ensure_prepared(ctx, L, precision, var);
   if (rc) return rc;
   const size_t LL = (size_t)L * L, rs = real_size(precision);
+  A.reserve(2 * Arena::round(3 * LL * rs) + 2 * Arena::round(sizeof(Solve)));
   void* planes = A.get(3 * LL * rs);
   void* spec = A.get(3 * LL * rs);
   double* dpath = (double*)A.get(4 * sizeof(double));
@@ -2374,22 +2698,12 @@ int epfft_serve_step(epfft_ctx* ctx, int32_t* n_running, int32_t* n_queued) {
   {
     // the records read with the step (a fired check is cleared by the
     // synchronous read), or read now when no class ran
-    CheckRec cr{};
-    if (checks_read) {
-      for (int i = 0; i < N_CHECK_UNITS && !cr.code; i++)
-        if (ctx->h_checks[i].code) cr = ctx->h_checks[i];
-      if (cr.code) {
-        CheckRec clr;
-        CK(read_check_all(&clr));
-      }
-    } else {
-      CK(read_check_all(&cr));
+    if (!checks_read) {
+      CK(enqueue_check_reads(ctx, ctx->stream));
+      CK(cudaStreamSynchronize(ctx->stream));
     }
-    if (cr.code) {
-      fprintf(stderr, "epfft: device self-check %d failed (index %lld, bound %lld, at %d)\n", cr.code,
-              (long long)cr.index, (long long)cr.bound, cr.where);
-      return EPFFT_ERR_CUDA;
-    }
+    rc = check_result(ctx);
+    if (rc) return rc;
   }
   for (ServeClass* k : live) {
     int64_t before = 0, after = 0;
