@@ -103,11 +103,17 @@ solve_onchip(Solve* __restrict__ solves, BatchCtl* bc, const C2<float>* __restri
   const C2<float>* rtw = s + O::OFF_RT;
   const C2<float>* ctw = s + O::OFF_CT;
   const C2<float>* oct = s + O::OFF_OCT;
-  __shared__ int s_phase;
+  // the CTA's copy of the solve: the state machine's fields and the pointers
+  // are read every phase, and from global memory each read costs an L2 trip
+  __shared__ __align__(16) unsigned char s_solve[sizeof(Solve)];
   __shared__ double tot[N_ACC];
   if (!ECHK(blockDim.x - 1, NT, 80)) return;
-  Solve& S = solves[blockIdx.x];
+  Solve& S = *reinterpret_cast<Solve*>(s_solve);
+  Solve* G = solves + blockIdx.x;
   const int tid = threadIdx.x;
+  for (int i = tid; i < (int)(sizeof(Solve) / 4); i += NT)
+    reinterpret_cast<unsigned*>(s_solve)[i] = reinterpret_cast<const unsigned*>(G)[i];
+  __syncthreads();
   copy_table<float, NT>(s + O::OFF_RT, tw + O::TB::off_row(0), O::RTW);
   copy_table<float, NT>(s + O::OFF_CT, tw + O::TB::off_col(0), O::CTW);
   copy_table<float, NT>(s + O::OFF_OCT, tw, O::OCT);
@@ -119,15 +125,13 @@ solve_onchip(Solve* __restrict__ solves, BatchCtl* bc, const C2<float>* __restri
   const int64_t bound = (int64_t)S.n_inc * ((int64_t)S.max_iter + 2) + 9;
   __syncthreads();
   for (int64_t step = 0;; step++) {
-    if (tid == 0) s_phase = *(volatile int32_t*)&S.phase;
-    __syncthreads();
-    const int phase = s_phase;
+    const int phase = S.phase;
     if (phase == PH_DONE) break;
     if (step >= bound) {
       if (tid == 0) atomicOr(&bc->timed_out, 1);
       break;
     }
-    const int cur = *(volatile int32_t*)&S.cur, inc = *(volatile int32_t*)&S.inc;
+    const int cur = S.cur, inc = S.inc;
     // ---- column phase (ITER): forward column transforms, Eq. 3, inverse ----
     if (phase == PH_ITER) {
       oc_transpose<L, true>(s);
@@ -254,13 +258,19 @@ solve_onchip(Solve* __restrict__ solves, BatchCtl* bc, const C2<float>* __restri
     if (phase == PH_ITER || phase == PH_INIT) {
       fft_seq<float, M, O::PS::RM_ROW, O::PS::FULL, 3 * L, NT, false>(s, rtw);
       oc_twist<L, true>(s, oct);
-      block_reduce_acc<NT>(acc, S.partials);
-      __syncthreads();
-      sum_partials<NT, 1>(S.partials, tot);
+      block_reduce_acc<NT>(acc, tot);  // the CTA's sums are the solve's
     }
     __syncthreads();
     if (tid == 0) finalize_solve<L>(S, phase, tot);
     __syncthreads();
+  }
+  if (tid == 0) {
+    G->phase = S.phase;
+    G->inc = S.inc;
+    G->iter = S.iter;
+    G->cur = S.cur;
+    G->status = S.status;
+    G->total_iters = S.total_iters;
   }
 }
 

@@ -615,6 +615,25 @@ __device__ __forceinline__ void sum_partials(const double* partials, double* out
   block_sum_f64<NWA>(v, out);
 }
 
+// x 2^-k, exactly, in integer instructions (an FP64 one takes 64 clocks of a
+// lone warp); results below the normal range by the multiplication.
+__device__ __forceinline__ double scale_down(double x, int k) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  if (e > k && e != 0x7ff) return __hiloint2double(hi - (k << 20), lo);
+  if (((hi & 0x7fffffff) | lo) == 0) return x;
+  return x * __hiloint2double((1023 - k) << 20, 0);
+}
+// x truncated to FP32 in integer instructions: 0 below its normal range,
+// infinity above (and for NaN).
+__device__ __forceinline__ float rough_float(double x) {
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+  if (e < 897) return 0.0f;
+  if (e > 1150) return CUDART_INF_F;
+  return __uint_as_float((unsigned)(hi & 0x80000000) | ((unsigned)((hi & 0x7fffffff) - 0x38000000) << 3) |
+                         (unsigned)__double2loint(x) >> 29);
+}
+
 // Last CTA of a solve's row pass: indicators of Sec. 2 and the state
 // machine.  Runs on one thread; A holds the sums of the partials (ITER).
 // The indicators are eta1 = sqrt(div2 / ss), eta2 = sqrt(dd / ss) and
@@ -626,6 +645,7 @@ __device__ __forceinline__ void sum_partials(const double* partials, double* out
 template <int L>
 __device__ __forceinline__ void finalize_solve(Solve& S, int phase, const double* A, bool record = true) {
   constexpr double inv = 1.0 / ((double)L * (double)L);  // exact: L is a power of two
+  constexpr int LG2 = 2 * ilog2c(L);
   if (phase == PH_INIT) {
     const double* E = S.path + 4 * S.inc;
     for (int c = 0; c < 4; c++) {
@@ -647,11 +667,32 @@ __device__ __forceinline__ void finalize_solve(Solve& S, int phase, const double
   // produced it); <eps> and the plastic count of iterate n come from the
   // previous pass
   double sig[4];
-  for (int c = 0; c < 4; c++) sig[c] = A[A_S11 + c] * inv;
-  const double div2 = A[A_DIV2] * inv, comp = A[A_COMP] * inv;
+  for (int c = 0; c < 4; c++) sig[c] = scale_down(A[A_S11 + c], LG2);
+  const double div2 = scale_down(A[A_DIV2], LG2), comp = scale_down(A[A_COMP], LG2);
   const int n = S.iter;
   S.total_iters += 1;
-  if (n >= 1) {
+  // Most iterates are far from the equilibrium test: when FP32 copies show the
+  // residual above the tolerance by more than their rounding can hide (0.1 %,
+  // and below any tolerance whose square leaves the FP32 range), the iterate
+  // is neither accepted nor non-finite, and the FP64 test (some 60 dependent
+  // instructions of one thread, 2 us) is left out.
+  bool far = false;
+  if (n >= 1 && n < S.max_iter) {
+    const float tol = rough_float(S.tol_eq), s0 = rough_float(sig[0]), s1 = rough_float(sig[1]),
+                s3 = rough_float(sig[3]), d = rough_float(S.eq_fixed_point ? S.comp_cur : div2);
+    float den = s0 * s0 + s1 * s1 + 2.0f * s3 * s3;
+    if (S.eq_fixed_point) {
+      const double* E = S.path + 4 * S.inc;
+      const float e0 = rough_float(E[0]), e1 = rough_float(E[1]), e2 = rough_float(E[2]), e3 = rough_float(E[3]);
+      den = e0 * e0 + e1 * e1 + e2 * e2 + 2.0f * e3 * e3;
+    }
+    const float ss = s0 * s0 + s1 * s1 + 2.0f * s3 * s3, r = rough_float(div2);
+    auto fin = [](double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; };
+    // finite, normal numbers only: the FP64 path decides the rest
+    far = fin(S.sig_prev[0]) && fin(S.sig_prev[1]) && fin(S.sig_prev[3]) && ss > 1e-30f && ss < 1e30f && den > 1e-30f && den < 1e30f && r < 1e30f && d < 1e30f &&
+          d > (1.001f * tol * tol + 1e-34f) * den && d > 1e-30f;
+  }
+  if (n >= 1 && !far) {
     const double* E = S.path + 4 * S.inc;
     double EE = E[0] * E[0] + E[1] * E[1] + E[2] * E[2] + 2.0 * E[3] * E[3];
     if (EE == 0.0) EE = 1.0;
@@ -711,7 +752,7 @@ __device__ __forceinline__ void finalize_solve(Solve& S, int phase, const double
   }
   for (int c = 0; c < 4; c++) {
     S.sig_prev[c] = sig[c];
-    S.epsm_next[c] = A[A_E11 + c] * inv;
+    S.epsm_next[c] = scale_down(A[A_E11 + c], LG2);
   }
   S.npl_next = A[A_NPL];
   S.comp_cur = comp;
