@@ -69,10 +69,11 @@ struct RsCfg {
   using P = RsPlan<L>;
   static constexpr int T = P::T;
   // columns per CTA: two (a tile) or more, 64 threads per CTA up to L = 512
-  // (eight CTAs per SM), 128 at L = 1024; one column above
-  // (two CTAs per SM at L = 4096; a CTA that held both columns of a tile
-  // would read whole sectors but fill the SM alone, which measured slower)
-  static constexpr int CPC = L <= 1024 ? (64 / T > 2 ? 64 / T : 2) : 1;
+  // (eight CTAs per SM), 128 at L = 1024; both columns of a two-column tile at
+  // L = 2048; one column at L = 4096 (two CTAs per SM; a CTA that held
+  // both columns of a tile would read whole sectors but fill the SM alone,
+  // which measured slower)
+  static constexpr int CPC = L <= 1024 ? (64 / T > 2 ? 64 / T : 2) : (L == 2048 && W == 2 ? 2 : 1);
   static constexpr int NT = CPC * T;
   // the two columns of a tile alternate lane by lane
   static constexpr bool INTER = CPC >= 2 && W == 2;

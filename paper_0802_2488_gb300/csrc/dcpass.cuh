@@ -178,9 +178,8 @@ __device__ __forceinline__ void st4(float* p, const float v[4]) {
 __device__ __forceinline__ void batch_arrive_dc(Solve* solves, int nb, BatchCtl* bc, cudaGraphConditionalHandle cond,
                                                 int use_cond, cudaGraphConditionalHandle rcond, int use_rcond) {
   __threadfence();
-  const unsigned total = gridDim.x * gridDim.y;
   const unsigned prev = atomicAdd(&bc->arrive, 1u);
-  if (prev == total - 1) {
+  if (prev == gridDim.y - 1) {
     __threadfence();
     int active = 0, waiting = 0;
     for (int i = 0; i < nb; i++) {
@@ -203,23 +202,28 @@ __device__ __forceinline__ void batch_arrive_dc(Solve* solves, int nb, BatchCtl*
   }
 }
 
-// Resident CTAs per SM asked of the compiler: at L = 512 four CTAs of 256
-// threads in tiling 0, two in tiling 1 (64 and 128 registers, no spills),
-// one elsewhere (the 1024- and 2048-point rows spill at 64).
+// Tile shape of the defect form's row pass.
 template <int L, int V>
-constexpr int dc_minb() { return L == 512 ? (V == 0 ? 4 : 2) : 1; }
+using DcCfg = Cfg<float, L, V + CFG_DEF>;
+// Resident CTAs per SM asked of the compiler: at L = 512 four CTAs of 256
+// threads in tiling 0, two in tiling 1 (64 and 128 registers, no spills), at
+// L = 128 and 256 of tiling 0 four of 128, one elsewhere (the 1024- and
+// 2048-point rows spill at 64).
+template <int L, int V>
+constexpr int dc_minb() { return L == 512 ? (V == 0 ? 4 : 2) : (V == 0 && (L == 128 || L == 256) ? 4 : 1); }
 
 template <int L, int V>
-__global__ void __launch_bounds__(Cfg<float, L, V>::NT_ROW, dc_minb<L, V>())
+__global__ void __launch_bounds__(DcCfg<L, V>::NT_ROW, dc_minb<L, V>())
 row_pass_dc(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<float>* __restrict__ tw,
             cudaGraphConditionalHandle cond, int use_cond, cudaGraphConditionalHandle rcond, int use_rcond) {
-  using C = Cfg<float, L, V>;
+  using C = DcCfg<L, V>;
   constexpr int RR = C::RR, NT = C::NT_ROW;
   constexpr int P = L >= NT ? L / NT : 1;
-  using IO = RowIO<float, L, V>;
+  using IO = RowIO<float, L, V + CFG_DEF>;
   extern __shared__ __align__(16) unsigned char smraw[];
   C2<float>* sp = reinterpret_cast<C2<float>*>(smraw);
   __shared__ bool s_last;
+  bool arrive = blockIdx.x == 0;  // of a solve that is skipped; else its last CTA
   if (!ECHK(gridDim.x - 1, L / RR, 70) || !ECHK(blockDim.x - 1, NT, 70)) return;
   Solve& S = solves[blockIdx.y];
   const volatile Solve& Sv = S;
@@ -470,6 +474,7 @@ row_pass_dc(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<float>* _
       s_last = prev == gridDim.x - 1;
     }
     __syncthreads();
+    arrive = s_last;
     if (s_last) {
       __shared__ double tot[N_ACC];
       __threadfence();
@@ -494,7 +499,7 @@ row_pass_dc(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<float>* _
       }
     }
   }
-  if (tid == 0) batch_arrive_dc(solves, nb, bc, cond, use_cond, rcond, use_rcond);
+  if (tid == 0 && arrive) batch_arrive_dc(solves, nb, bc, cond, use_cond, rcond, use_rcond);
 }
 
 // Refresh, forward half (FP64 tiling V; grid (L / RR, solves)), for the

@@ -195,7 +195,7 @@ bool supported(int L, int prec) {
 int shape(int L, int prec, int var, PassShape* sh) {
   bool ok;
   if (var == ONCHIP_VARIANT) ok = prec == EPFFT_FP32 && onchip_supported(L) && pass_shape<float>(L, 0, sh);
-  else if (prec == EPFFT_FP32_DEFECT) ok = var < N_DEF_VARIANTS && pass_shape<float>(L, var, sh);
+  else if (prec == EPFFT_FP32_DEFECT) ok = var < N_DEF_VARIANTS && pass_shape_def(L, var, sh);
   else ok = prec == EPFFT_FP32 ? pass_shape<float>(L, var, sh) : pass_shape<double>(L, var, sh);
   return ok ? EPFFT_OK : EPFFT_ERR_UNSUPPORTED;
 }

@@ -15,13 +15,35 @@ static cudaError_t prepare_def_L() {
   constexpr int V = EPFFT_VAR;
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(row_pass_dc<L, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)Cfg<float, L, V>::ROW_SMEM)) != cudaSuccess)
+                                (int)DcCfg<L, V>::ROW_SMEM)) != cudaSuccess)
     return e;
   if ((e = cudaFuncSetAttribute(dc_ref_forward<L, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)Cfg<double, L, V>::ROW_SMEM)) != cudaSuccess)
     return e;
   return cudaFuncSetAttribute(dc_ref_inverse<L, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)Cfg<double, L, V>::ROW_SMEM);
+}
+
+template <>
+bool pass_shape_def_v<EPFFT_VAR>(int L, PassShape* o) {
+  switch (L) {
+#define X(n)                                     \
+  case n: {                                      \
+    using C = DcCfg<n, EPFFT_VAR>;               \
+    o->rows_per_cta = C::RR;                     \
+    o->tile_w = C::W;                            \
+    o->row_ctas = n / C::RR;                     \
+    o->col_ctas = (n / 2) / C::W;                \
+    o->nt_row = C::NT_ROW;                       \
+    o->nt_col = C::NT_COL;                       \
+    o->row_smem = C::ROW_SMEM;                   \
+    o->col_smem = C::COL_SMEM;                   \
+    return true;                                 \
+  }
+    EPFFT_DEF_FOR_L(X)
+#undef X
+    default: return false;
+  }
 }
 
 template <>
@@ -41,7 +63,7 @@ cudaError_t launch_row_def_v<EPFFT_VAR>(int L, int nb, cudaStream_t s, Solve* so
   switch (L) {
 #define X(n)                                                                                             \
   case n: {                                                                                              \
-    using C = Cfg<float, n, EPFFT_VAR>;                                                                  \
+    using C = DcCfg<n, EPFFT_VAR>;                                                                       \
     row_pass_dc<n, EPFFT_VAR><<<dim3(n / C::RR, nb), C::NT_ROW, C::ROW_SMEM, s>>>(                      \
         solves, nb, bc, reinterpret_cast<const C2<float>*>(tw), cond, use_cond, rcond, use_rcond);       \
     return cudaGetLastError();                                                                           \

@@ -55,6 +55,8 @@ cudaError_t check_record_v(void** out);
 // V: forward row half, the FP64 column pass, inverse row half, the sums).
 constexpr int N_DEF_VARIANTS = 2;
 template <int V>
+bool pass_shape_def_v(int L, PassShape* out);  // its row pass's shape
+template <int V>
 cudaError_t prepare_def_v(int L);
 template <int V>
 cudaError_t launch_row_def_v(int L, int nb, cudaStream_t s, Solve* solves, BatchCtl* bc, const void* tw,
@@ -71,6 +73,14 @@ cudaError_t read_check_def_v(CheckRec* out);
 template <int V>
 cudaError_t check_record_def_v(void** out);
 
+template <int D = 0>  // a template, so that the variants may be specialised after it
+inline bool pass_shape_def(int L, int var, PassShape* out) {
+  switch (var) {
+    case 0: return pass_shape_def_v<0>(L, out);
+    case 1: return pass_shape_def_v<1>(L, out);
+    default: return false;
+  }
+}
 template <int D = 0>  // a template, so that the variants may be specialised after it
 inline cudaError_t prepare_def(int L, int var) {
   switch (var) {

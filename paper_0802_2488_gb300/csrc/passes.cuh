@@ -37,9 +37,15 @@ namespace epfft {
 //          runs rely on the L2 to merge neighbouring CTAs' accesses).
 // Shared memory of a pass: its sequences (padded, fft.cuh), then its stage
 // table, then (row pass) the twist octant.
-template <typename T, int L, int V = 0>
+// V + CFG_DEF is tiling V with the row shape of the defect form, whose row pass
+// holds more per pixel (same tile width and plans, so the same spectrum
+// layout and column pass).
+constexpr int CFG_DEF = 4;
+template <typename T, int L, int VV = 0>
 struct Cfg {
   static constexpr bool F64 = sizeof(T) == 8;
+  static constexpr int V = VV % CFG_DEF;
+  static constexpr bool DEF = VV >= CFG_DEF;
   static constexpr int M = L / 2;
   using PS = PlanSel<T, L, V>;
   using PR = typename PS::PR;
@@ -47,8 +53,16 @@ struct Cfg {
   using TB = Tables<T, L>;
   static constexpr int RM_ROW = PS::RM_ROW, RM_COL = PS::RM_COL;
   static constexpr bool FULL = PS::FULL;
-  // rows per row-pass CTA
-  static constexpr int RR = V == 0 ? (F64 ? 2 : (L <= 256 ? 2 : (L == 512 ? 4 : (L <= 2048 ? 8 : 4))))
+  // rows per row-pass CTA.  FP32 tiling 0 (batches): small CTAs, several per SM
+  // at 64 registers a thread, so that one CTA's tile wait and barriers overlap
+  // the others' work; measured for batches of 64 (L = 1024: 16, 2048: 4),
+  // rows x threads: L = 128 4 x 128 36 us (2 x 128 57; 8 x 128 31, but slower for
+  // the few lattices a serving class often runs), L = 256 4 x 128 91
+  // (2 x 256 205, 16 x 256 150), L = 512 4 x 256 299 (8 x 512 337), L = 1024
+  // 2 x 256 341 (8 x 512 432, 4 x 512 368), L = 2048 2 x 512 446 (8 x 512 462).
+  static constexpr int RR0 = L <= 64 ? 2 : (L <= 512 || L == 4096 ? 4 : 2);
+  static constexpr int RR0_DEF = L <= 64 ? 2 : (L == 2048 ? 8 : 4);
+  static constexpr int RR = V == 0 ? (F64 ? 2 : (DEF ? RR0_DEF : RR0))
                                    : (F64 ? (L <= 256 || L == 4096 ? 1 : 2) : (L <= 256 ? 1 : 2));
   // columns per column-pass CTA (= tile width of the spectrum layout)
   static constexpr int W0 = V == 0 ? (F64 ? (L <= 256 ? 1 : (L <= 1024 ? 2 : 1))
@@ -56,19 +70,19 @@ struct Cfg {
                                    : (F64 ? 1 : (L <= 256 ? 1 : (L <= 1024 ? 2 : (L <= 2048 ? 1 : 2))));
   static constexpr int W = W0 < M ? W0 : M;
   static constexpr int NTMAX = V == 0 ? 512 : 256;
-  // resident CTAs per SM asked of the compiler: FP32 variant 1 (at most 128
-  // registers per thread at 256 threads), the FP32 L = 512 row pass of
-  // variant 0 (four CTAs of 4 rows and 256 threads at 64 registers, no
-  // spills: 307 us at 64 x L = 512 against 337 us for two CTAs of 8 rows
-  // and 512 threads, whose 16-warp barriers and tile waits overlapped
-  // less) and the FP32 column
+  // resident CTAs per SM asked of the compiler: FP32 variant 1 at most 128
+  // registers per thread at 256 threads, the FP32 rows of variant 0 from
+  // L = 128 to 2048 64 (1024 threads per SM), and the FP32 column
   // passes of the narrow tiles of variant 0 at L = 512 .. 2048: 768 threads
   // per SM at L = 512 (85 registers, no spills), three CTAs of 384 at
   // L = 1024 and 2048 (56 registers), so that the CTAs of an SM overlap
   // their loads with the others' transforms
-  static constexpr int MINB_ROW = !F64 && (V == 1 || L == 512) ? (V == 0 ? 4 : 2) : 1;
   static constexpr int NT_ROW0 = F64 ? (L > 512 ? 256 : (L < 128 ? L : 128))
-                                     : (L <= 256 ? L : (V == 0 && L == 512 ? 256 : NTMAX));
+                                     : (V == 1 ? (L <= 256 ? L : NTMAX)
+                                               : (L <= 128 ? L
+                                                           : (L == 256 ? 128
+                                                                       : (L == 512 || (L == 1024 && !DEF) ? 256 : 512))));
+  static constexpr int MINB_ROW = F64 ? 1 : (V == 1 ? 2 : (L >= 128 && L <= 2048 ? 1024 / NT_ROW0 : 1));
   static constexpr int NT_ROW = NT_ROW0 < 32 ? 32 : NT_ROW0;
   static constexpr int NT_COL0 = ((3 * W * L / RM_COL + 31) / 32) * 32;
   // 256 threads for the FP64 L = 4096 column: at 512 the 128 registers a
@@ -458,7 +472,7 @@ struct RowIO {
   // table; the octant follows it.
   static __device__ __forceinline__ const C2<T>* load_tables(C2<T>* sp, const C2<T>* __restrict__ tab) {
     C2<T>* stw = sp + SZ;
-    copy_table<T, NT>(stw, tab + C::TB::off_row(V), C::ROW_TW);
+    copy_table<T, NT>(stw, tab + C::TB::off_row(C::V), C::ROW_TW);
     copy_table<T, NT>(stw + C::ROW_TW, tab, C::TB::OCT);
     return stw;
   }
@@ -760,14 +774,16 @@ __device__ __forceinline__ void finalize_solve(Solve& S, int phase, const double
   S.cur = 1 - S.cur;
 }
 
-// After every CTA of the row pass: the last one decides whether the
-// device-side loop runs another step (condition of the graph's while node).
+// Once per solve of the row pass's launch, by the last CTA of the solve (one of
+// a finished solve's): the last solve's decides whether the device-side loop
+// runs another step (condition of the graph's while node).  (Counting every
+// CTA instead held each one for another fence and atomic round trip, all at
+// one address.)
 __device__ __forceinline__ void batch_arrive(Solve* solves, int nb, BatchCtl* bc,
                                              cudaGraphConditionalHandle cond, int use_cond) {
   __threadfence();
-  const unsigned total = gridDim.x * gridDim.y;
   const unsigned prev = atomicAdd(&bc->arrive, 1u);
-  if (prev == total - 1) {
+  if (prev == gridDim.y - 1) {
     __threadfence();
     int active = 0, waiting = 0;
     for (int i = 0; i < nb; i++) {
@@ -1077,6 +1093,7 @@ row_pass(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<T>* __restri
   extern __shared__ __align__(16) unsigned char smraw[];
   C2<T>* sp = reinterpret_cast<C2<T>*>(smraw);
   __shared__ bool s_last;
+  bool arrive = blockIdx.x == 0;  // of a finished solve; else its last CTA
 
   // Every index of the pass is in range when the grid has L / RR CTAs per
   // solve (see RowIO::where; pixel x = (r0 + r) L + x1 < L^2 for x1 < L).
@@ -1101,6 +1118,7 @@ row_pass(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<T>* __restri
       s_last = prev == gridDim.x - 1;
     }
     __syncthreads();
+    arrive = s_last;
     if (s_last) {
       __shared__ double tot[N_ACC];
       __threadfence();
@@ -1114,7 +1132,7 @@ row_pass(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<T>* __restri
       }
     }
   }
-  if (tid == 0) batch_arrive(solves, nb, bc, cond, use_cond);
+  if (tid == 0 && arrive) batch_arrive(solves, nb, bc, cond, use_cond);
 }
 
 // ---------------------------------------------------------------------------

@@ -315,6 +315,7 @@ row_pass_rs(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<float>* _
   constexpr int M = CF::M, T = CF::T, RR = CF::RR, NT = CF::NT, R1 = P::R1, K1 = P::E / R1;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ bool s_last;
+  bool arrive = blockIdx.x == 0;  // of a finished solve; else its last CTA
   if (!ECHK(blockDim.x - 1, NT, 50) || !ECHK(gridDim.x - 1, L / RR, 50)) return;
   Solve& S = solves[blockIdx.y];
   const volatile Solve& Sv = S;
@@ -436,6 +437,7 @@ row_pass_rs(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<float>* _
       s_last = prev == gridDim.x - 1;
     }
     __syncthreads();
+    arrive = s_last;
     if (s_last) {
       __shared__ double tot[N_ACC];
       __threadfence();
@@ -449,7 +451,7 @@ row_pass_rs(Solve* __restrict__ solves, int nb, BatchCtl* bc, const C2<float>* _
       }
     }
   }
-  if (tid == 0) batch_arrive(solves, nb, bc, cond, use_cond);
+  if (tid == 0 && arrive) batch_arrive(solves, nb, bc, cond, use_cond);
 }
 
 // Row transforms alone (tiling variant 2): the forward transform of three
