@@ -62,10 +62,15 @@ struct Cfg {
   // 2 x 256 341 (8 x 512 432, 4 x 512 368), L = 2048 2 x 512 446 (8 x 512 462).
   static constexpr int RR0 = L <= 64 ? 2 : (L <= 512 || L == 4096 ? 4 : 2);
   static constexpr int RR0_DEF = L <= 64 ? 2 : (L == 2048 ? 8 : 4);
-  static constexpr int RR = V == 0 ? (F64 ? 2 : (DEF ? RR0_DEF : RR0))
+  // FP64 tiling 0: one row of 128 threads at L = 512, four CTAs per SM at 128
+  // registers (8 x L = 512: 324 us; two rows, two CTAs at 191 registers 424;
+  // 2 x 256 threads 358, 4 x 256 351), two rows of 256 at L = 1024 (232 us;
+  // 285 at one CTA per SM), one of 256 at 2048 (940 us; two rows 1070).
+  static constexpr int RR64 = L == 512 || L == 2048 ? 1 : 2;
+  static constexpr int RR = V == 0 ? (F64 ? RR64 : (DEF ? RR0_DEF : RR0))
                                    : (F64 ? (L <= 256 || L == 4096 ? 1 : 2) : (L <= 256 ? 1 : 2));
   // columns per column-pass CTA (= tile width of the spectrum layout)
-  static constexpr int W0 = V == 0 ? (F64 ? (L <= 256 ? 1 : (L <= 1024 ? 2 : 1))
+  static constexpr int W0 = V == 0 ? (F64 ? 1
                                           : (L == 2048 ? 1 : 2))
                                    : (F64 ? 1 : (L <= 256 ? 1 : (L <= 1024 ? 2 : (L <= 2048 ? 1 : 2))));
   static constexpr int W = W0 < M ? W0 : M;
@@ -82,14 +87,17 @@ struct Cfg {
                                                : (L <= 128 ? L
                                                            : (L == 256 ? 128
                                                                        : (L == 512 || (L == 1024 && !DEF) ? 256 : 512))));
-  static constexpr int MINB_ROW = F64 ? 1 : (V == 1 ? 2 : (L >= 128 && L <= 2048 ? 1024 / NT_ROW0 : 1));
+  static constexpr int MINB_ROW = F64 ? (V == 0 && L >= 256 && L <= 2048 ? 512 / NT_ROW0 : 1) : (V == 1 ? 2 : (L >= 128 && L <= 2048 ? 1024 / NT_ROW0 : 1));
   static constexpr int NT_ROW = NT_ROW0 < 32 ? 32 : NT_ROW0;
   static constexpr int NT_COL0 = ((3 * W * L / RM_COL + 31) / 32) * 32;
-  // 256 threads for the FP64 L = 4096 column: at 512 the 128 registers a
-  // thread spill (3.75 ms against 2.74)
-  static constexpr int NTMAX_COL = F64 && L == 4096 ? 256 : NTMAX;
+  // 256 threads at most for FP64 columns: at 512 the 128 registers of a
+  // thread spill at L = 4096 (3.75 ms against 2.74), and one column on 256
+  // threads three times per SM (80 registers) beats two on 512 at L = 512
+  // (8 x L = 512: 205 us against 330)
+  static constexpr int NTMAX_COL = F64 ? 256 : NTMAX;
   static constexpr int NT_COL = NT_COL0 < 32 ? 32 : (NT_COL0 > NTMAX_COL ? NTMAX_COL : NT_COL0);
-  static constexpr int MINB_COL = F64 ? 1
+  // FP64: 768 threads per SM up to L = 512, 512 at L = 1024 (244 -> 170 us)
+  static constexpr int MINB_COL = F64 ? (L <= 512 ? 768 / NT_COL : (L == 1024 ? 2 : 1))
                                       : V == 1 ? 2 : (L == 512 ? 768 / NT_COL : (L == 1024 || L == 2048 ? 3 : 1));
   // sequences transformed per call: the largest divisor of the sequence
   // count that keeps at most 16 elements per thread and stage
