@@ -305,6 +305,44 @@ __device__ __forceinline__ void green_apply(C2<T> k1, C2<T> k2, T lam0, T mu0, T
   p12 = T(-0.5) * (k1 * v2 + k2 * v1);
 }
 
+// The symmetrized operator (DG1) at symbols k1 = k(m1), k2 = k(m2).  G(-q) is
+// the complex conjugate of G(q) (k(-q) = -k(q)*), so the mean over the four
+// sign choices is the mean of Re G(q1, q2) and D Re G(-q1, q2) D, D =
+// diag(1, 1, -1): a real symmetric coupling of the spectrum.  With c = k1* k2
+// (c = -k1 k2 for the mirrored operator), M = the adjugate of N and the
+// factor -1/det of green_apply,
+//   11,11: N22 |k1|^2    22,22: N11 |k2|^2    11,22: -(lm cr^2 + d ci^2)
+//   11,12: cr (N22 - lm |k1|^2)   22,12: cr (N11 - lm |k2|^2)
+//   12,12 (halved): N11 |k1|^2 + N22 |k2|^2 - 2 (lm cr^2 - d ci^2),
+// lm = lam0 + mu0, d = lam0 - mu0, N12 = lm cr + i d ci.  About 80
+// instructions a frequency against 300 for four applications (FP32 L = 1024: 79
+// -> 65 us an iteration).
+template <typename T>
+__device__ __forceinline__ void dg1_apply(C2<T> k1, C2<T> k2, T lam0, T mu0, T scale, C2<T>& p11, C2<T>& p22,
+                                          C2<T>& p12) {
+  const T a1 = norm2(k1), a2 = norm2(k2), K2 = a1 + a2;
+  const T lm = lam0 + mu0, d = lam0 - mu0, mk2 = mu0 * K2;
+  const T N11 = lm * a1 + mk2, N22 = lm * a2 + mk2;
+  const T d0 = (lam0 + T(2) * mu0) * mk2 * K2, db = T(4) * lam0 * mu0;
+  const T rr = k1.re * k2.re, ii = k1.im * k2.im, ri = k1.re * k2.im, ir = k1.im * k2.re;
+  const T cr = rr + ii, ci = ri - ir, xr = ii - rr, xi = -(ri + ir);  // c, and c of the mirrored operator
+  const T cr2 = cr * cr, ci2 = ci * ci, xr2 = xr * xr, xi2 = xi * xi;
+  // half of each operator; the mirrored one's 12 couplings change sign
+  const T h = T(-0.5) * scale;
+  const T f = h * rcp(d0 + db * ci2), g = h * rcp(d0 + db * xi2);
+  const T fg = f + g, s = f * cr - g * xr;
+  const T u = f * (lm * cr2) + g * (lm * xr2), v = f * (d * ci2) + g * (d * xi2);
+  const T g11 = fg * (N22 * a1), g22 = fg * (N11 * a2), gx = -(u + v);
+  const T g1 = s * (N22 - lm * a1), g2 = s * (N11 - lm * a2);
+  const T g12 = T(0.5) * (fg * (N11 * a1 + N22 * a2)) - (u - v);
+  const C2<T> e11 = g11 * p11 + gx * p22 + g1 * p12;
+  const C2<T> e22 = gx * p11 + g22 * p22 + g2 * p12;
+  const C2<T> e12 = T(0.5) * (g1 * p11 + g2 * p22) + g12 * p12;
+  p11 = e11;
+  p22 = e22;
+  p12 = e12;
+}
+
 // Displacement of Sec. 2 at frequency (m1, m2) != 0 from the strain
 // spectrum (e11, e22, e12) in (p11, p22, p12): with k^2 = k1^2 + k2^2,
 //   u1 = -(i / k^2) { k1 [e11 - e22] + 2 k2 e12 },
@@ -391,22 +429,7 @@ __device__ __forceinline__ void green_op(int mode, const C2<T>* __restrict__ kta
     return;
   }
   // GM_DG1
-  const int n1 = (L - m1) & (L - 1), n2 = (L - m2) & (L - 1);  // indices of -q1, -q2
-  C2<T> b11 = a11, b22 = a22, b12 = a12;
-  green_apply(ktab[m1], ktab[m2], lam0, mu0, scale, b11, b22, b12);
-  C2<T> s11 = b11, s22 = b22, s12 = b12;
-  b11 = a11, b22 = a22, b12 = a12;
-  green_apply(ktab[n1], ktab[n2], lam0, mu0, scale, b11, b22, b12);
-  s11 = s11 + b11, s22 = s22 + b22, s12 = s12 + b12;
-  b11 = a11, b22 = a22, b12 = T(-1) * a12;
-  green_apply(ktab[n1], ktab[m2], lam0, mu0, scale, b11, b22, b12);
-  s11 = s11 + b11, s22 = s22 + b22, s12 = s12 - b12;
-  b11 = a11, b22 = a22, b12 = T(-1) * a12;
-  green_apply(ktab[m1], ktab[n2], lam0, mu0, scale, b11, b22, b12);
-  s11 = s11 + b11, s22 = s22 + b22, s12 = s12 - b12;
-  p11 = T(0.25) * s11;
-  p22 = T(0.25) * s22;
-  p12 = T(0.25) * s12;
+  dg1_apply(ktab[m1], ktab[m2], lam0, mu0, scale, p11, p22, p12);
 }
 
 }  // namespace epfft
