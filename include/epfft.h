@@ -211,7 +211,9 @@ int epfft_solve(epfft_ctx *ctx, const epfft_problem *problem, const epfft_path *
  * epfft_autotune or epfft_set_tiling) runs instead as one kernel launch, one
  * CTA per problem, on a stream forked from the context's stream, while the
  * graph of the other groups runs.  records[i] is a host array of
- * paths[i].n_inc entries; fields may be NULL or an array of n.  The
+ * paths[i].n_inc entries; fields may be NULL or an array of n.  A call of one
+ * group of small lattices runs as one cooperative launch instead of the graph,
+ * with the same results.  The
  * arithmetic of each problem does not depend on the others in the batch. */
 int epfft_solve_batch(epfft_ctx *ctx, int32_t n, const epfft_problem *problems,
                       const epfft_path *paths, epfft_record *const *records,

@@ -1361,9 +1361,11 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
   // counts; then one read-back of the solve states, the control blocks, the
   // records, the counts and the self-check records
   int launches = 1;  // the gathering of the self-check records
+  // (a caller's buffer off the 16-byte boundary is copied after the read-back)
+  auto aligned = [&](int i) { return ((uintptr_t)eps_out[i] & 15) == 0; };
   if (eps_out)
     for (int i = 0; i < n; i++)
-      if (eps_out[i]) {
+      if (eps_out[i] && aligned(i)) {
         Batch& B = Bs[where[i]];
         const int64_t words = (int64_t)B.L * B.L * (int64_t)real_size(B.prec) / 4;
         accepted_strain_kernel<<<(unsigned)std::min<int64_t>((words + 255) / 256, 152 * 16), 256, 0, c->stream>>>(
@@ -1473,13 +1475,16 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
     const Solve& S = B.h_solves[j];
     if (S.phase != PH_DONE && S.status == 0) return EPFFT_ERR_DEVICE_TIMEOUT;
     if (records) std::memcpy(records[i], R.data(), sizeof(Record) * (size_t)B.n_inc[j]);
+    if (eps_out && eps_out[i] && !aligned(i))
+      CK(cudaMemcpyAsync(eps_out[i], S.eps[S.cur], 4 * (size_t)B.L * B.L * real_size(B.prec),
+                         cudaMemcpyDeviceToDevice, c->stream));
     if (iter_rec) std::memcpy(&iter_rec[i], &R[B.n_inc[j] - 1], sizeof(Record));
     for (int k = 0; k < B.n_inc[j]; k++) {
       if (R[k].status == 2) status = EPFFT_ERR_NUMERIC;
       else if (R[k].status == 1 && status == EPFFT_OK) status = EPFFT_NOT_CONVERGED;
     }
   }
-  if (fields) CK(cudaStreamSynchronize(c->stream));
+  if (fields || eps_out) CK(cudaStreamSynchronize(c->stream));
   if (cs != c->stream) CK(cudaStreamSynchronize(cs));
   return status;
 }

@@ -53,3 +53,21 @@ def test_mixed_call_equals_resident_alone():
         for i in range(2):
             _same(B.epfft_solve_batch(ctx, probs[i:i + 1], paths[i:i + 1], fields=True),
                   (rc, recs[i:i + 1], fs[i:i + 1]))
+
+
+def test_iterate_accepts_a_strain_off_the_16_byte_boundary():
+    """The accepted strain is written back by a kernel of 16-byte words, or by a
+    copy where the caller's buffer does not start on such a boundary."""
+    import torch
+    from paper_0802_2488_gb300 import binding as B
+    L = 32
+    base = torch.rand(4 * L * L + 1, device="cuda", generator=torch.Generator("cuda").manual_seed(3)) * 0.5
+    a = base[:-1].clone().view(L, L, 4)
+    b = torch.empty(4 * L * L + 1, device="cuda")[1:].view(L, L, 4)
+    b.copy_(a)
+    assert b.data_ptr() % 16 == 4
+    with B.Context(0) as ctx:
+        prob = B.Problem(L=L, precision="fp32", void_fraction=0.2, seed=1)
+        for t in (a, b):
+            B.epfft_iterate(ctx, prob, [0.3, 0.2, 0.0, 0.1], t, 3)
+    assert torch.equal(a, b)
