@@ -505,7 +505,8 @@ def roofline(precision, L, nb, col_ms, row_ms, peak, peak_source, tiling=None):
     reference data read 40, mask 1), column pass 24.
     FP64 (FP64 ALU): flops per pixel, row pass 15 log2 L + 60 (row
     transforms, local step), column pass 15 log2 L + 25 (column transforms,
-    Green operator)."""
+    Green operator); the transforms' flops are done in 64-bit integers, so the
+    fraction of the FP64 peak can exceed 1."""
     n = L * L * nb
     lg = int(np.log2(L))
     if precision in ("fp32", "fp32_defect"):
@@ -536,7 +537,8 @@ def roofline(precision, L, nb, col_ms, row_ms, peak, peak_source, tiling=None):
             "frac": d["frac"], "traffic": tr[0] if tr else None, "traffic_note": note,
             "peak_source": peak_source, "passes": passes,
             "timing": "epfft_time_passes: CUDA events around each launch on the context stream, mean of the "
-                      "timed launches, the same launch shape as the solve"}
+                      "timed launches, the same launch shape as the solve" +
+                      ("; the transforms' flops of the count are done in 64-bit integers" if bound == "alu" else "")}
 
 
 def solve_line(B, ctx, stream, flush, torch, name, precision, cap, steps, warmup, e2e_steps, local, ws,

@@ -23,10 +23,11 @@
 // every operation).  A NaN or infinity in the block makes every output of the
 // block NaN (as one in a sequence does to the sequence's outputs).
 //
-// Measured (8 x L = 512, CUDA events): column pass 581 -> 330 us; row pass
-// 787 -> 631 us, and 416 us with the twists in fixed point too and the pixel
-// step of local_step64 (what is left on the FP64 pipe is the Green operator
-// and the pixel step); L = 4096: 5.69 -> 2.74 ms and 7.83 -> 4.15 ms.
+// Measured (8 x L = 512, CUDA events): column pass 581 -> 330 us, row pass
+// 787 -> 631 us, 416 with the twists in fixed point too and the pixel step of
+// local_step64, and 205 and 330 us with the CTA shapes this left room for
+// (Cfg in passes.cuh); what is left on the FP64 pipe is the Green operator and
+// the pixel step.  L = 4096: 5.69 -> 2.74 ms and 7.83 -> 4.15 ms.
 // Against long double: projection at L = 64, 256 1.8e-16, 1.9e-16 relative
 // (FP64 butterflies 3.2e-16, 3.6e-16), 20 iterations at L = 256 7.0e-16
 // (1.25e-15).
