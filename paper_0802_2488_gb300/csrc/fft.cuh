@@ -306,47 +306,90 @@ __device__ __forceinline__ void fft_stages(C2<T>* s, const C2<T>* __restrict__ t
   }
 }
 
-// Largest of a value over the CTA's NT threads (every thread calls it; it
-// holds one barrier, and the caller another one before the next call).
+// Block exponents of the sequences a CTA holds (double sequences, fft64.cuh):
+// wm: largest high words by groups of 32 numbers or butterflies, em: the
+// exponents.  One per CTA (and NT).
+struct __align__(16) SeqScratch {
+  unsigned wm[64];
+  int em[8];
+};
 template <int NT>
-__device__ __forceinline__ unsigned block_max_u32(unsigned x) {
-  __shared__ unsigned wm[NT / 32];
-  x = __reduce_max_sync(0xffffffffu, x);
-  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = x;
-  __syncthreads();
-  unsigned m = wm[0];
+__device__ __forceinline__ SeqScratch& seq_scratch() {
+  __shared__ SeqScratch s;
+  return s;
+}
+// Largest value over aligned groups of n lanes (a power of two; the warp from 32
+// on).  Every lane calls it.  Groups of 8 and 16 take a warp reduction each,
+// which do not wait for one another as the steps of a butterfly would.
+template <int n>
+__device__ __forceinline__ unsigned lanes_max(unsigned x) {
+  if constexpr (n >= 32) {
+    return __reduce_max_sync(0xffffffffu, x);
+  } else if constexpr (n >= 8) {
+    const int own = (threadIdx.x & 31) / n;
+    unsigned m = 0;
 #pragma unroll
-  for (int i = 1; i < NT / 32; i++) m = max(m, wm[i]);
+    for (int k = 0; k < 32 / n; k++) {
+      const unsigned y = __reduce_max_sync(0xffffffffu, own == k ? x : 0u);
+      if (own == k) m = y;
+    }
+    return m;
+  } else {
+#pragma unroll
+    for (int o = n / 2; o > 0; o >>= 1) x = max(x, __shfl_xor_sync(0xffffffffu, x, o));
+    return x;
+  }
+}
+// Largest of n slots (n a power of two, slots 4 n bytes aligned up to 16).
+template <int n>
+__device__ __forceinline__ unsigned slots_max(const unsigned* w) {
+  unsigned m = 0;
+  if constexpr (n % 4 == 0) {
+#pragma unroll
+    for (int i = 0; i < n; i += 4) {
+      const uint4 a = *reinterpret_cast<const uint4*>(w + i);
+      m = max(m, max(max(a.x, a.y), max(a.z, a.w)));
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < n; i++) m = max(m, w[i]);
+  }
   return m;
 }
 
 // The Stockham stage in fixed point (double sequences, fft64.cuh): the same
 // butterflies, addresses and barriers as stockham_stage.  The first stage
-// finds the block exponent of the NSEQ sequences and converts, the last one
-// rounds to doubles.  RENORM: before the stage the integers are shifted up to
+// finds the block exponent of each of the NSEQ sequences (into em[], shared)
+// and converts, the last one rounds to doubles.  A sequence's largest number
+// is found by its warp where a stage has at most 32 butterflies per sequence,
+// else through a slot per warp and step.  RENORM: before the stage the
+// integers are shifted up to
 // the 62 bits again.  The stages' divisions cost sequences of a few large
 // numbers (the spectrum of a field with a large mean) up to log2 N bits;
 // shifting up before each stage that would take them to seven (six before a
 // radix-16 stage) keeps the
 // rounding below that of FP64 butterflies for them too (projection with a
 // mean strain at L = 1024 against long double: 8.3e-16 without, 2.0e-16 with,
-// 4.1e-16 for FP64 butterflies).  emax: the block exponent.
-// IN_INT: the sequences already hold integers made with emax (moduli below
-// 2^62.5 / R of the first stage); OUT_INT: they are left as integers.
-template <int N, int RM, bool FULL, int NSEQ, int NT, int K, bool INV, bool IN_INT, bool OUT_INT>
-__device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>* __restrict__ tw, int& emax) {
+// 4.1e-16 for FP64 butterflies).
+// IN_INT: the sequences already hold integers made with em[] (moduli below
+// 2^62.5 / R of the first stage); OUT_INT: they are left as integers, em[]
+// theirs.  The outputs are those of the transform times 2^XLG.
+template <int N, int RM, bool FULL, int NSEQ, int NT, int K, bool INV, bool IN_INT, bool OUT_INT, int XLG>
+__device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>* __restrict__ tw, int* em) {
   using P = FftPlan<N, RM, FULL>;
   constexpr int R = P::radix(K), NS = P::ns(K), LR = ilog2c(R);
   constexpr int NJ = N / R, NBF = NSEQ * NJ, KB = (NBF + NT - 1) / NT, SP = seq_stride<N>();
   constexpr bool FIRST = K == 0, LAST = K == P::NSTAGES - 1, RENORM = !FIRST && ilog2c(NS) + LR >= (LR == 4 ? 6 : 7);
-  constexpr bool CONVERT = FIRST && !IN_INT;
+  constexpr bool CONVERT = FIRST && !IN_INT, SLOTS = (CONVERT || RENORM) && NJ > 32;
+  static_assert(!SLOTS || NBF / 32 <= (int)(sizeof(SeqScratch::wm) / sizeof(unsigned)), "slots");
   C2<i64>* z = reinterpret_cast<C2<i64>*>(s);
   C2<i64> v[KB][R];
   const int tid = threadIdx.x;
-  unsigned mx = 0;
+  unsigned mx[KB];
 #pragma unroll
   for (int q = 0; q < KB; q++) {
     const int g = tid + q * NT;
+    mx[q] = 0;
     if (NBF % NT == 0 || g < NBF) {
       const int j = g % NJ, sq = g / NJ;
       const int rb = sq * SP + (NJ >= 32 ? pad32(j) : j);
@@ -354,35 +397,52 @@ __device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>
       for (int r = 0; r < R; r++) {
         v[q][r] = z[rb + read_off<N, R, NS>(r)];
         const int hr = (int)(v[q][r].re >> 32), hi = (int)(v[q][r].im >> 32);
-        if constexpr (CONVERT) mx = max(mx, max((unsigned)hr & 0x7fffffffu, (unsigned)hi & 0x7fffffffu));
-        if constexpr (RENORM) mx = max(mx, (unsigned)max(hr ^ (hr >> 31), hi ^ (hi >> 31)));
+        if constexpr (CONVERT) mx[q] = max(mx[q], max((unsigned)hr & 0x7fffffffu, (unsigned)hi & 0x7fffffffu));
+        if constexpr (RENORM) mx[q] = max(mx[q], (unsigned)max(hr ^ (hr >> 31), hi ^ (hi >> 31)));
       }
     }
   }
-  int sh = 0;
   if constexpr (CONVERT || RENORM) {
-    mx = block_max_u32<NT>(mx);
-    if constexpr (CONVERT) {
-      emax = block_exp(mx);
-    } else {
-      sh = max(__clz((int)mx) - 2, 0);
-      if (emax >= 2047) sh = 0;
-      emax -= sh;
+#pragma unroll
+    for (int q = 0; q < KB; q++) mx[q] = lanes_max<NJ>(mx[q]);
+  }
+  if constexpr (SLOTS) {
+    unsigned* wm = seq_scratch<NT>().wm;
+#pragma unroll
+    for (int q = 0; q < KB; q++) {
+      const int g = tid + q * NT;
+      if ((tid & 31) == 0 && (NBF % NT == 0 || g < NBF)) wm[g / 32] = mx[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < KB; q++) {
+      const int g = tid + q * NT;
+      if (NBF % NT == 0 || g < NBF) mx[q] = slots_max<NJ / 32>(wm + (g / NJ) * (NJ / 32));
     }
   }
+  int eo[KB];  // block exponent of the outputs (LAST)
 #pragma unroll
   for (int q = 0; q < KB; q++) {
     const int g = tid + q * NT;
     if (NBF % NT == 0 || g < NBF) {
-      const int j = g % NJ;
+      const int j = g % NJ, sq = g / NJ;
       if constexpr (CONVERT) {
+        const int e = block_exp(mx[q]);
+        if (j == 0 && (!LAST || OUT_INT)) em[sq] = e;
+        eo[q] = e;
 #pragma unroll
         for (int r = 0; r < R; r++) {
-          v[q][r].re = to_fixed<LR>(__longlong_as_double(v[q][r].re), emax);
-          v[q][r].im = to_fixed<LR>(__longlong_as_double(v[q][r].im), emax);
+          v[q][r].re = to_fixed<LR>(__longlong_as_double(v[q][r].re), e);
+          v[q][r].im = to_fixed<LR>(__longlong_as_double(v[q][r].im), e);
         }
-      } else if constexpr (!FIRST) {
+      } else {
+        if constexpr (LAST && !OUT_INT) eo[q] = em[sq];
+      }
+      if constexpr (!FIRST) {
         if constexpr (RENORM) {
+          const int sh = max(__clz((int)mx[q]) - 2, 0);
+          if constexpr (LAST && !OUT_INT) eo[q] -= sh;
+          else if (j == 0) em[sq] -= sh;
 #pragma unroll
           for (int r = 0; r < R; r++) {
             v[q][r].re = (i64)((unsigned long long)v[q][r].re << sh);
@@ -399,7 +459,7 @@ __device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>
       Bfly64<R, INV>::run(v[q]);
     }
   }
-  if constexpr (!(CONVERT || RENORM)) __syncthreads();  // else block_max_u32's barrier followed every read
+  if constexpr (!SLOTS) __syncthreads();  // else the slots' barrier followed every read
 #pragma unroll
   for (int q = 0; q < KB; q++) {
     const int g = tid + q * NT;
@@ -407,10 +467,11 @@ __device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>
       const int j = g % NJ, sq = g / NJ;
       const int jm = j % NS, a = (j / NS) * NS * R;
       const int wb = sq * SP + (N < 32 ? a + jm : (NS <= 32 ? a + (a >> 5) + jm : pad32(a + jm)));
+      constexpr int LG = ilog2c(N) + XLG;
 #pragma unroll
       for (int r = 0; r < R; r++) {
         const int i = wb + write_off<N, R, NS>(r);
-        if constexpr (LAST && !OUT_INT) s[i] = mk(from_fixed<ilog2c(N)>(v[q][r].re, emax), from_fixed<ilog2c(N)>(v[q][r].im, emax));
+        if constexpr (LAST && !OUT_INT) s[i] = mk(from_fixed<LG>(v[q][r].re, eo[q]), from_fixed<LG>(v[q][r].im, eo[q]));
         else z[i] = v[q][r];
       }
     }
@@ -418,11 +479,12 @@ __device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>
   __syncthreads();
 }
 
-template <int N, int RM, bool FULL, int NSEQ, int NT, bool INV, bool IN_INT = false, bool OUT_INT = false, int K = 0>
-__device__ __forceinline__ void fft_stages64(C2<double>* s, const C2<double>* __restrict__ tw, int& emax) {
+template <int N, int RM, bool FULL, int NSEQ, int NT, bool INV, bool IN_INT = false, bool OUT_INT = false, int XLG = 0,
+          int K = 0>
+__device__ __forceinline__ void fft_stages64(C2<double>* s, const C2<double>* __restrict__ tw, int* em) {
   if constexpr (K < FftPlan<N, RM, FULL>::NSTAGES) {
-    stockham_stage64<N, RM, FULL, NSEQ, NT, K, INV, IN_INT, OUT_INT>(s, tw, emax);
-    fft_stages64<N, RM, FULL, NSEQ, NT, INV, IN_INT, OUT_INT, K + 1>(s, tw, emax);
+    stockham_stage64<N, RM, FULL, NSEQ, NT, K, INV, IN_INT, OUT_INT, XLG>(s, tw, em);
+    fft_stages64<N, RM, FULL, NSEQ, NT, INV, IN_INT, OUT_INT, XLG, K + 1>(s, tw, em);
   }
 }
 
@@ -433,8 +495,8 @@ __device__ __forceinline__ void fft_stages64(C2<double>* s, const C2<double>* __
 template <typename T, int N, int RM, bool FULL, int NSEQ, int NT, bool INV>
 __device__ __forceinline__ void fft_seq(C2<T>* s, const C2<T>* __restrict__ tw) {
   if constexpr (sizeof(T) == 8) {
-    int emax = 0;
-    fft_stages64<N, RM, FULL, NSEQ, NT, INV>(s, tw, emax);
+    static_assert(NSEQ <= (int)(sizeof(SeqScratch::em) / sizeof(int)), "exponents");
+    fft_stages64<N, RM, FULL, NSEQ, NT, INV>(s, tw, seq_scratch<NT>().em);
   } else {
     fft_stages<T, N, RM, FULL, NSEQ, NT, INV>(s, tw);
   }

@@ -4,9 +4,12 @@
 // scheduler), a 64-bit integer add (two instructions) about every 1.5 and a
 // 32 x 32 + 64 bit multiply-add every 2.1 clocks (measured).  A transform is
 // additions and multiplications by numbers of modulus 1, so it is done in
-// 64-bit fixed point on a block exponent: the group of sequences that one
-// call transforms is read as doubles, their largest exponent found, and each
-// number x held as the integer x 2^B of a common B.  A stage of radix R
+// 64-bit fixed point on a block exponent: each sequence is read as doubles,
+// its largest exponent found, and each number x of it held as the integer
+// x 2^B of a common B.  (One B for all sequences of a call is not enough:
+// components that do not couple, or rows, far below the largest would lose
+// bits that FP64 butterflies, whose error follows the sequence's own norm, keep.
+// A component 1e-10 of the others: 6e-8 of its norm against 1e-16.)  A stage of radix R
 // multiplies by its twiddles scaled by 2^64 / R and keeps the upper 64 bits
 // of the 128-bit product, which divides by R, so no sum can overflow
 // whatever the data are:
@@ -16,12 +19,12 @@
 //   modulus <= 2^62.5 again.
 //
 // The last stage's integers are rounded to doubles.  Precision: an input is
-// held to 2^-60 of the block's largest number, each stage rounds to the last
+// held to 2^-60 of the sequence's largest number, each stage rounds to the last
 // bit of numbers whose RMS falls by sqrt(R) a stage from 2^60 or so, which
 // leaves an error of 2^-55 (N = 512) to 2^-53 (N = 4096) of the output's RMS,
 // below that of the FP64 butterflies it replaces (their 53 bits are rounded at
-// every operation).  A NaN or infinity in the block makes every output of the
-// block NaN (as one in a sequence does to the sequence's outputs).
+// every operation).  A NaN or infinity in a sequence makes every output of it
+// NaN.
 //
 // Measured (8 x L = 512, CUDA events): column pass 581 -> 330 us, row pass
 // 787 -> 631 us, 416 with the twists in fixed point too and the pixel step of
@@ -159,10 +162,13 @@ EPFFT_HD double make_double(unsigned long long b) {
 }
 
 // Block exponent of the largest high word mx (sign bit cleared): the biased
-// exponent, at least 65 (blocks below 2^-957 lose their last bits).
+// exponent, at least 65 (sequences below 2^-957 lose their last bits), or
+// FIX_NAN for an infinity or a NaN (far above any exponent, so that the shifts
+// between stages leave it one).
+constexpr int FIX_NAN = 1 << 20;
 EPFFT_HD int block_exp(unsigned mx) {
   const int e = (int)(mx >> 20);
-  return e < 65 ? 65 : e;
+  return e < 65 ? 65 : (e >= 2047 ? FIX_NAN : e);
 }
 // x 2^(B - emax + 1022), B = 62 - G: below 2^B in modulus for |x| <
 // 2^(emax - 1022).
@@ -179,7 +185,7 @@ EPFFT_HD i64 to_fixed(double x, int emax) {
 }
 // v 2^(emax - 1084 + LG) rounded to the nearest double: the output of a
 // length 2^LG transform of numbers made by to_fixed (every stage divides by
-// its radix).  Underflow gives 0, overflow infinity, emax = 2047 NaN.
+// its radix).  Underflow gives 0, overflow infinity, FIX_NAN NaN.
 template <int LG>
 EPFFT_HD double from_fixed(i64 v, int emax) {
   const unsigned sg = (unsigned)((unsigned long long)v >> 32) & 0x80000000u;
@@ -194,8 +200,8 @@ EPFFT_HD double from_fixed(i64 v, int emax) {
   unsigned long long b = (n >> 11) + ((n >> 10) & 1ull);
   b += (unsigned long long)(unsigned)(E - 1) << 52;
   if (a == 0 || E <= 0) b = 0;
-  if (E >= 2047) b = 0x7ff0000000000000ull;
-  if (emax >= 2047) b = 0x7ff8000000000000ull;
+  // (with FIX_NAN, E is as large for every v)
+  if (E >= 2047) b = (unsigned long long)(emax >= FIX_NAN / 2 ? 0x7ff80000u : 0x7ff00000u) << 32;
   return make_double(b | (unsigned long long)sg << 32);
 }
 

@@ -297,49 +297,114 @@ struct RowIO {
     }
   }
   // Double precision: the twists work on the fixed-point numbers of the
-  // transforms (fft64.cuh).  The inverse one finds the tile's block exponent,
-  // converts and leaves integers of a quarter of Z (moduli below 2^62.5 / R0
-  // of the first stage) for fft<true>; the forward one takes the integers
-  // fft<false> leaves (block exponent s_em[group]) and writes doubles.
+  // transforms (fft64.cuh), with a block exponent per sequence (em, shared).
+  // The inverse one converts and leaves integers of a quarter of Z (moduli below
+  // 2^62.5 / R0 of the first stage) for fft<true>; the forward one takes the
+  // integers fft<false> leaves and writes doubles.
   static constexpr int LG_R0 = ilog2c(C::PR::radix(0));
   static constexpr int NG = NSEQ / C::G_R;  // transform calls per tile
-  static __device__ __forceinline__ int c2r_twist64(C2<T>* sp, const C2<T>* __restrict__ oct) {
-    unsigned mx = 0;
-    for (int i = threadIdx.x; i < NSEQ * M; i += NT) {
-      const int q = (i / M) * SP + pad32(i % M);
-      if (!ECHK(q, SZ, 38)) continue;
-      const C2<T> z = sp[q];
-      mx = max(mx, max((unsigned)hi_word(z.re) & 0x7fffffffu, (unsigned)hi_word(z.im) & 0x7fffffffu));
-    }
-    const int emax = block_exp(block_max_u32<NT>(mx));
-    auto pair = [&](int k, int sq0, int ds) {
-      const int kk = M - k;
-      const int ik = pad32(k), ikk = pad32(kk);  // 0 < k, kk < M
+  static_assert(sizeof(T) == 4 || NSEQ <= (int)(sizeof(SeqScratch::em) / sizeof(int)), "exponents");
+  static __device__ __forceinline__ unsigned high_max(const C2<T>& z) {
+    return max((unsigned)hi_word(z.re) & 0x7fffffffu, (unsigned)hi_word(z.im) & 0x7fffffffu);
+  }
+  // Elements k (a) and M - k (b) of Z as integers, into s, and element 0.
+  static __device__ __forceinline__ void c2r_pair64(C2<T>* s, int k, const Tw64& wk, int e, const C2<T>& a, const C2<T>& b) {
+    const int kk = M - k;
+    C2<i64>* z = reinterpret_cast<C2<i64>*>(s);
+    const i64 ar = to_fixed<LG_R0>(a.re, e), ai = to_fixed<LG_R0>(a.im, e);
+    const i64 br = to_fixed<LG_R0>(b.re, e), bi = to_fixed<LG_R0>(b.im, e);
+    i64 tr = ar - br, ti = ai + bi;
+    cmul_hi<true>(tr, ti, wk);
+    const i64 sr = rshift<2>(ar + br), si = rshift<2>(ai - bi);
+    z[pad32(k)] = mk(sr - ti, si + tr);
+    if (kk != k) z[pad32(kk)] = mk(sr + ti, tr - si);
+  }
+  static __device__ __forceinline__ void c2r_zero64(C2<T>* s, int e) {
+    const i64 a = to_fixed<LG_R0>(s[0].re, e), b = to_fixed<LG_R0>(s[0].im, e);
+    reinterpret_cast<C2<i64>*>(s)[0] = mk(rshift<2>(a + b), rshift<2>(a - b));
+  }
+  static __device__ __forceinline__ void c2r_twist64(C2<T>* sp, const C2<T>* __restrict__ oct, int* em) {
+    constexpr int HK = M / 2;
+    unsigned* wm = seq_scratch<NT>().wm;
+    const int tid = threadIdx.x;
+    if constexpr (NT >= HK) {
+      // a thread's pairs stay in registers while the exponents are found
+      constexpr int DS = NT / HK, NQ = (NSEQ + DS - 1) / DS;
+      static_assert(HK <= 32 || NSEQ * (HK / 32) <= (int)(sizeof(SeqScratch::wm) / sizeof(unsigned)), "slots");
+      const int k = 1 + tid % HK, ik = pad32(k), ikk = pad32(M - k);
       const Tw64 wk = twist_tw64<L>(oct, k);
-      for (int sq = sq0; sq < NSEQ; sq += ds) {
-        C2<T>* s = sp + sq * SP;
-        if (!ECHK(sq * SP + ikk, SZ, 38) || !ECHK(sq * SP + ik, SZ, 38)) continue;
-        C2<i64>* z = reinterpret_cast<C2<i64>*>(s);
-        const i64 ar = to_fixed<LG_R0>(s[ik].re, emax), ai = to_fixed<LG_R0>(s[ik].im, emax);
-        const i64 br = to_fixed<LG_R0>(s[ikk].re, emax), bi = to_fixed<LG_R0>(s[ikk].im, emax);
-        i64 tr = ar - br, ti = ai + bi;
-        cmul_hi<true>(tr, ti, wk);
-        const i64 sr = rshift<2>(ar + br), si = rshift<2>(ai - bi);
-        z[ik] = mk(sr - ti, si + tr);
-        if (kk != k) z[ikk] = mk(sr + ti, tr - si);
+      C2<T> a[NQ], b[NQ];
+      unsigned mx[NQ];
+#pragma unroll
+      for (int i = 0; i < NQ; i++) {
+        const int sq = tid / HK + i * DS;
+        mx[i] = 0;
+        if (sq >= NSEQ || !ECHK(sq * SP + ikk, SZ, 38) || !ECHK(sq * SP + ik, SZ, 38)) continue;
+        a[i] = sp[sq * SP + ik];
+        b[i] = sp[sq * SP + ikk];
+        mx[i] = max(high_max(a[i]), high_max(b[i]));
+        if (k == 1) mx[i] = max(mx[i], high_max(sp[sq * SP]));
       }
-    };
-    visit_pairs(pair);
-    for (int sq = threadIdx.x; sq < NSEQ; sq += NT) {
-      C2<T>* s = sp + sq * SP;
-      const i64 a = to_fixed<LG_R0>(s[0].re, emax), b = to_fixed<LG_R0>(s[0].im, emax);
-      reinterpret_cast<C2<i64>*>(s)[0] = mk(rshift<2>(a + b), rshift<2>(a - b));
+#pragma unroll
+      for (int i = 0; i < NQ; i++) mx[i] = lanes_max<HK>(mx[i]);
+      if constexpr (HK > 32) {
+#pragma unroll
+        for (int i = 0; i < NQ; i++) {
+          const int sq = tid / HK + i * DS;
+          if ((tid & 31) == 0 && sq < NSEQ) wm[sq * (HK / 32) + (tid % HK) / 32] = mx[i];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < NQ; i++) {
+          const int sq = tid / HK + i * DS;
+          if (sq < NSEQ) mx[i] = slots_max<HK / 32>(wm + sq * (HK / 32));
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < NQ; i++) {
+        const int sq = tid / HK + i * DS;
+        if (sq >= NSEQ || !ECHK(sq * SP + ikk, SZ, 38) || !ECHK(sq * SP + ik, SZ, 38)) continue;
+        const int e = block_exp(mx[i]);
+        c2r_pair64(sp + sq * SP, k, wk, e, a[i], b[i]);
+        if (k == 1) {
+          c2r_zero64(sp + sq * SP, e);
+          em[sq] = e;
+        }
+      }
+    } else {
+      // the exponents first, by a slot per sequence and warp
+      constexpr int SPS = NT / 32;
+      static_assert(M % NT == 0 && NSEQ * SPS <= (int)(sizeof(SeqScratch::wm) / sizeof(unsigned)), "slots");
+#pragma unroll
+      for (int sq = 0; sq < NSEQ; sq++) {
+        unsigned mx = 0;
+#pragma unroll
+        for (int j = 0; j < M / NT; j++) {
+          const int q = sq * SP + pad32(j * NT + tid);
+          if (ECHK(q, SZ, 38)) mx = max(mx, high_max(sp[q]));
+        }
+        mx = lanes_max<32>(mx);
+        if ((tid & 31) == 0) wm[sq * SPS + (tid >> 5)] = mx;
+      }
+      __syncthreads();
+      // every warp writes them all, and reads only its own before the next barrier
+      if ((tid & 31) < NSEQ) em[tid & 31] = block_exp(slots_max<SPS>(wm + (tid & 31) * SPS));
+      __syncwarp();
+      visit_pairs([&](int k, int sq0, int ds) {
+        const int ik = pad32(k), ikk = pad32(M - k);  // 0 < k, M - k < M
+        const Tw64 wk = twist_tw64<L>(oct, k);
+        for (int sq = sq0; sq < NSEQ; sq += ds) {
+          C2<T>* s = sp + sq * SP;
+          if (!ECHK(sq * SP + ikk, SZ, 38) || !ECHK(sq * SP + ik, SZ, 38)) continue;
+          c2r_pair64(s, k, wk, em[sq], s[ik], s[ikk]);
+        }
+      });
+      for (int sq = tid; sq < NSEQ; sq += NT) c2r_zero64(sp + sq * SP, em[sq]);
     }
-    return emax;
   }
   // half of X(k) (see r2c_twist), so that the sums stay below 2^63
-  static __device__ __forceinline__ void r2c_twist64(C2<T>* sp, const C2<T>* __restrict__ oct, const int* s_em) {
-    constexpr int LG = ilog2c(M);
+  static __device__ __forceinline__ void r2c_twist64(C2<T>* sp, const C2<T>* __restrict__ oct, const int* em) {
+    constexpr int LG = ilog2c(M) + 1;
     auto pair = [&](int k, int sq0, int ds) {
       const int kk = M - k;
       const int ik = pad32(k), ikk = pad32(kk);  // 0 < k, kk < M
@@ -347,21 +412,21 @@ struct RowIO {
       for (int sq = sq0; sq < NSEQ; sq += ds) {
         C2<T>* s = sp + sq * SP;
         if (!ECHK(sq * SP + ikk, SZ, 38) || !ECHK(sq * SP + ik, SZ, 38)) continue;
-        const int em = s_em[NG == 1 ? 0 : sq / C::G_R] + 1;
+        const int e = em[sq];
         const C2<i64> a = reinterpret_cast<C2<i64>*>(s)[ik], b = reinterpret_cast<C2<i64>*>(s)[ikk];
         i64 tr = (a.re >> 1) - (b.re >> 1), ti = (a.im >> 1) + (b.im >> 1);
         cmul_half(tr, ti, wk);
         const i64 sr = rshift<1>((a.re >> 1) + (b.re >> 1)), si = rshift<1>((a.im >> 1) - (b.im >> 1));
-        s[ik] = mk(from_fixed<LG>(sr + ti, em), from_fixed<LG>(si - tr, em));
-        if (kk != k) s[ikk] = mk(from_fixed<LG>(sr - ti, em), from_fixed<LG>(-si - tr, em));
+        s[ik] = mk(from_fixed<LG>(sr + ti, e), from_fixed<LG>(si - tr, e));
+        if (kk != k) s[ikk] = mk(from_fixed<LG>(sr - ti, e), from_fixed<LG>(-si - tr, e));
       }
     };
     visit_pairs(pair);
     for (int sq = threadIdx.x; sq < NSEQ; sq += NT) {
       C2<T>* s = sp + sq * SP;
-      const int em = s_em[NG == 1 ? 0 : sq / C::G_R] + 1;
+      const int e = em[sq];
       const C2<i64> z = reinterpret_cast<C2<i64>*>(s)[0];
-      s[0] = mk(from_fixed<LG>((z.re >> 1) + (z.im >> 1), em), from_fixed<LG>((z.re >> 1) - (z.im >> 1), em));
+      s[0] = mk(from_fixed<LG>((z.re >> 1) + (z.im >> 1), e), from_fixed<LG>((z.re >> 1) - (z.im >> 1), e));
     }
   }
   // Spectrum tile (loaded, after a barrier) -> real rows, and back.  Both
@@ -369,13 +434,12 @@ struct RowIO {
   // followed by one of the caller's.
   static __device__ __forceinline__ void rows_inverse(C2<T>* sp, const C2<T>* __restrict__ stw) {
     if constexpr (sizeof(T) == 8) {
-      const int emax = c2r_twist64(sp, octant(stw)) + 2;
+      int* em = seq_scratch<NT>().em;
+      c2r_twist64(sp, octant(stw), em);
       __syncthreads();
 #pragma unroll 1
-      for (int g = 0; g < NG; g++) {
-        int em = emax;
-        fft_stages64<M, C::RM_ROW, C::FULL, C::G_R, NT, true, true, false>(sp + g * C::G_R * SP, stw, em);
-      }
+      for (int g = 0; g < NG; g++)
+        fft_stages64<M, C::RM_ROW, C::FULL, C::G_R, NT, true, true, false, 2>(sp + g * C::G_R * SP, stw, em + g * C::G_R);
     } else {
       c2r_twist(sp, octant(stw));
       __syncthreads();
@@ -384,15 +448,11 @@ struct RowIO {
   }
   static __device__ __forceinline__ void rows_forward(C2<T>* sp, const C2<T>* __restrict__ stw) {
     if constexpr (sizeof(T) == 8) {
-      __shared__ int s_em[NG];
+      int* em = seq_scratch<NT>().em;
 #pragma unroll 1
-      for (int g = 0; g < NG; g++) {
-        int em = 0;
-        fft_stages64<M, C::RM_ROW, C::FULL, C::G_R, NT, false, false, true>(sp + g * C::G_R * SP, stw, em);
-        if (threadIdx.x == 0) s_em[g] = em;
-      }
-      __syncthreads();
-      r2c_twist64(sp, octant(stw), s_em);
+      for (int g = 0; g < NG; g++)
+        fft_stages64<M, C::RM_ROW, C::FULL, C::G_R, NT, false, false, true>(sp + g * C::G_R * SP, stw, em + g * C::G_R);
+      r2c_twist64(sp, octant(stw), em);
     } else {
       fft<false>(sp, stw);
       r2c_twist(sp, octant(stw));
