@@ -430,10 +430,19 @@ __device__ __forceinline__ void stockham_stage64(C2<double>* s, const C2<double>
         const int e = block_exp(mx[q]);
         if (j == 0 && (!LAST || OUT_INT)) em[sq] = e;
         eo[q] = e;
+        int ec = e;
+#pragma unroll 1
+        for (; ec < FIX_LOW; ec += 64) {
+#pragma unroll
+          for (int r = 0; r < R; r++) {
+            v[q][r].re = __double_as_longlong(lift64(__longlong_as_double(v[q][r].re)));
+            v[q][r].im = __double_as_longlong(lift64(__longlong_as_double(v[q][r].im)));
+          }
+        }
 #pragma unroll
         for (int r = 0; r < R; r++) {
-          v[q][r].re = to_fixed<LR>(__longlong_as_double(v[q][r].re), e);
-          v[q][r].im = to_fixed<LR>(__longlong_as_double(v[q][r].im), e);
+          v[q][r].re = to_fixed<LR>(__longlong_as_double(v[q][r].re), ec);
+          v[q][r].im = to_fixed<LR>(__longlong_as_double(v[q][r].im), ec);
         }
       } else {
         if constexpr (LAST && !OUT_INT) eo[q] = em[sq];

@@ -162,14 +162,19 @@ EPFFT_HD double make_double(unsigned long long b) {
 }
 
 // Block exponent of the largest high word mx (sign bit cleared): the biased
-// exponent, at least 65 (sequences below 2^-957 lose their last bits), or
-// FIX_NAN for an infinity or a NaN (far above any exponent, so that the shifts
-// between stages leave it one).
-constexpr int FIX_NAN = 1 << 20;
+// exponent, at least 1, or FIX_NAN for an infinity or a NaN (far above any
+// exponent, so that the shifts between stages leave it one).  to_fixed takes
+// exponents from FIX_LOW on: numbers of a sequence below that (2^-957) are
+// converted as 2^64 times themselves (lift64, exact) on an exponent 64 larger;
+// the callers write this as a loop, which the compiler leaves a branch (as
+// predicated FP64 instructions it cost every sequence 5 %).  Results below the
+// normal range (2^-1022) become zero.
+constexpr int FIX_NAN = 1 << 20, FIX_LOW = 65;
 EPFFT_HD int block_exp(unsigned mx) {
   const int e = (int)(mx >> 20);
-  return e < 65 ? 65 : (e >= 2047 ? FIX_NAN : e);
+  return e < 1 ? 1 : (e >= 2047 ? FIX_NAN : e);
 }
+EPFFT_HD double lift64(double x) { return x * 18446744073709551616.0; }
 // x 2^(B - emax + 1022), B = 62 - G: below 2^B in modulus for |x| <
 // 2^(emax - 1022).
 template <int G>

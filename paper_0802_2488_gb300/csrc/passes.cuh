@@ -308,8 +308,13 @@ struct RowIO {
     return max((unsigned)hi_word(z.re) & 0x7fffffffu, (unsigned)hi_word(z.im) & 0x7fffffffu);
   }
   // Elements k (a) and M - k (b) of Z as integers, into s, and element 0.
-  static __device__ __forceinline__ void c2r_pair64(C2<T>* s, int k, const Tw64& wk, int e, const C2<T>& a, const C2<T>& b) {
+  static __device__ __forceinline__ void c2r_pair64(C2<T>* s, int k, const Tw64& wk, int e, C2<T> a, C2<T> b) {
     const int kk = M - k;
+#pragma unroll 1
+    for (; e < FIX_LOW; e += 64) {
+      a = mk(lift64(a.re), lift64(a.im));
+      b = mk(lift64(b.re), lift64(b.im));
+    }
     C2<i64>* z = reinterpret_cast<C2<i64>*>(s);
     const i64 ar = to_fixed<LG_R0>(a.re, e), ai = to_fixed<LG_R0>(a.im, e);
     const i64 br = to_fixed<LG_R0>(b.re, e), bi = to_fixed<LG_R0>(b.im, e);
@@ -320,7 +325,10 @@ struct RowIO {
     if (kk != k) z[pad32(kk)] = mk(sr + ti, tr - si);
   }
   static __device__ __forceinline__ void c2r_zero64(C2<T>* s, int e) {
-    const i64 a = to_fixed<LG_R0>(s[0].re, e), b = to_fixed<LG_R0>(s[0].im, e);
+    C2<T> z = s[0];
+#pragma unroll 1
+    for (; e < FIX_LOW; e += 64) z = mk(lift64(z.re), lift64(z.im));
+    const i64 a = to_fixed<LG_R0>(z.re, e), b = to_fixed<LG_R0>(z.im, e);
     reinterpret_cast<C2<i64>*>(s)[0] = mk(rshift<2>(a + b), rshift<2>(a - b));
   }
   static __device__ __forceinline__ void c2r_twist64(C2<T>* sp, const C2<T>* __restrict__ oct, int* em) {

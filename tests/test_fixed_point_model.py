@@ -88,8 +88,13 @@ static void run(std::vector<double>& x, int RM) {
   }
   int em = block_exp(mx);
   std::vector<C2<i64>> z(N);
+  const bool low = em < FIX_LOW;
+  const int ec = low ? em + 64 : em;
   for (int i = 0; i < N; i++) {
-    auto f = [&](double v) { return L0 == 1 ? in<1>(v, em) : L0 == 2 ? in<2>(v, em) : L0 == 3 ? in<3>(v, em) : in<4>(v, em); };
+    auto f = [&](double v) {
+      if (low) v = lift64(v);
+      return L0 == 1 ? in<1>(v, ec) : L0 == 2 ? in<2>(v, ec) : L0 == 3 ? in<3>(v, ec) : in<4>(v, ec);
+    };
     z[i].re = f(x[2 * i]);
     z[i].im = f(x[2 * i + 1]);
   }
@@ -173,7 +178,7 @@ def test_transform_against_long_double(model, N, RM, inverse):
     amp[0] = top * (1 + 1j)
     tol = 4 * 2.0 ** -53 * np.log2(N)
     for name, x in (("white", white), ("mean", mean), ("pixel", pixel), ("amplitude", amp),
-                    ("large", 1e300 * white), ("small", 1e-250 * white)):
+                    ("large", 1e300 * white), ("small", 1e-250 * white), ("smallest", 2.0 ** -1000 * white)):
         assert _err(model(x, RM, inverse), _dft(x, inverse)) < tol, name
 
 
