@@ -65,22 +65,29 @@ __device__ __forceinline__ Mat<T> make_mat(const Solve& S) {
   return m;
 }
 
-// 1/sqrt(x) for x > 0 in normal FP32 range.  FP32: the hardware estimate.
+// 1/sqrt(x) for normal x > 0.  FP32: the hardware estimate.
 // FP64: the FP32 estimate refined by two Newton-Raphson steps
 // y <- y (3/2 - x y^2 / 2), each of which squares the relative error
 // (2e-7 -> 1e-13 -> below FP64 rounding), so that the kernel uses FP64 FMAs
-// only.
+// only.  The steps work on x / 2^(2k) in [1, 4) (exact), since x is a squared
+// strain or stress in the caller's units and may lie outside the FP32 range;
+// below the normal FP64 range the result is NaN.
 template <typename T>
 __device__ __forceinline__ T rsq(T x);
 template <>
 __device__ __forceinline__ float rsq<float>(float x) { return rsqrtf(x); }
+// (2 k) << 20 for the high word of x = m 2^(2k), 1 <= m < 4
+__device__ __forceinline__ int even_exp(int hi) { return (hi - 0x3ff00000) & (int)0xffe00000; }
 template <>
 __device__ __forceinline__ double rsq<double>(double x) {
-  double y = (double)rsqrtf((float)x);
-  const double h = 0.5 * x;
+  const int hi = __double2hiint(x), k2 = even_exp(hi);
+  const double m = __hiloint2double(hi - k2, __double2loint(x));
+  double y = (double)rsqrtf((float)m);
+  const double h = 0.5 * m;
   y = y * fma(-h * y, y, 1.5);
   y = y * fma(-h * y, y, 1.5);
-  return y;
+  y = __hiloint2double(__double2hiint(y) - (k2 >> 1), __double2loint(y));
+  return hi >= 0x00100000 && hi < 0x7ff00000 ? y : CUDART_NAN;
 }
 
 // 1/x for x > 0 in normal FP32 range.  FP32: the fast reciprocal (within
@@ -258,11 +265,13 @@ __device__ __forceinline__ bool local_step64(const double s[4], double e11, doub
   double sc = is_void ? m.inv_2mu0 : m.inv_2mumu0, gsc = is_void ? 0.0 : m.gsc_el;
   double pb = is_void ? -1.0 : m.pb_el;
   if (pl) {
-    // 1 / sqrt(h): FP32 estimate (2^-22), one third-order step
-    const int hi = __double2hiint(h);
-    const float f = __int_as_float((int)((unsigned)(hi - 0x38000000) << 3 | (unsigned)__double2loint(h) >> 29));
+    // 1 / sqrt(h): FP32 estimate (2^-22) of h / 2^(2k) in [1, 4), one
+    // third-order step; NaN below the normal range (see rsq)
+    const int hi = __double2hiint(h), k2 = even_exp(hi);
+    const float f = __int_as_float((int)((unsigned)(hi - k2 - 0x38000000) << 3 | (unsigned)__double2loint(h) >> 29));
     const int fb = __float_as_int(rsqrtf(f));
-    double y = __hiloint2double((fb >> 3) + 0x38000000, fb << 29);
+    double y = __hiloint2double((fb >> 3) + 0x38000000 - (k2 >> 1), fb << 29);
+    if (hi < 0x00100000) y = CUDART_NAN;
     const double r = fma(-(h * y), y, 1.0);
     y = fma(y * r, fma(0.375, r, 0.5), y);
     gsc = m.ylim_r2 * y;  // sqrt(2/3) Y / |tau'|
