@@ -135,8 +135,7 @@ __global__ void vp_relabel_kernel(const uint8_t* __restrict__ mask, const int32_
     const int64_t b = img * n;
     int32_t last = -1, cnt = 0;
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
-      const int32_t r = lab[b + x];
-      const int32_t f = r < 0 ? -1 : vp.final_root[b + vp.target[b + r]];
+      const int32_t f = vp_cluster(lab[b + x], vp.target + b, vp.final_root + b, n);
       if (out) out[b + x] = f;
       if (f < 0) continue;
       if (f != last) {

@@ -33,6 +33,17 @@ cudaError_t launch_avg5(const T* in, T* out, int L, cudaStream_t s);
 // vp.stats the counts.  n_voids_dev: void pixels of the mask.
 cudaError_t launch_vp_attach(const uint8_t* mask, const int32_t* lab, int32_t* out, int64_t n_img, int L,
                              const VpScratch& vp, const int32_t* n_voids_dev, cudaStream_t s);
+// Final cluster of a pixel labelled r by the first labelling, -1 for none.
+// Every index is checked: where a bounded chase of the labelling gave up (the
+// error flag is read after these kernels), r may be no root, and the scratch
+// there was never written.
+__host__ __device__ inline int32_t vp_cluster(int32_t r, const int32_t* target, const int32_t* final_root, int64_t n) {
+  if (r < 0 || r >= n) return -1;
+  const int32_t t = target[r];
+  if (t < 0 || t >= n) return -1;
+  const int32_t f = final_root[t];
+  return f >= 0 && f < n ? f : -1;
+}
 // out(x) = [(2/3) e'_ij e'_ij]^(1/2) of a strain field (Fig. 1), e' the 3D
 // deviator of (11, 22, 33, 12), e'_12 counted twice.
 template <typename T>
