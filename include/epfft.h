@@ -213,7 +213,10 @@ int epfft_solve(epfft_ctx *ctx, const epfft_problem *problem, const epfft_path *
  * graph of the other groups runs.  records[i] is a host array of
  * paths[i].n_inc entries; fields may be NULL or an array of n.  A call of one
  * group of small lattices runs as one cooperative launch instead of the graph,
- * with the same results.  The
+ * with the same results (the graph where the device refuses that launch).  The
+ * cooperative launch starts once all of its CTAs, up to the whole GPU, can be
+ * resident together: a kernel of the caller's that holds SMs until the solve
+ * is done must not run beside it.  The
  * arithmetic of each problem does not depend on the others in the batch. */
 int epfft_solve_batch(epfft_ctx *ctx, int32_t n, const epfft_problem *problems,
                       const epfft_path *paths, epfft_record *const *records,

@@ -904,20 +904,25 @@ int resident_ctas(epfft_ctx* c, int L, int prec, int var, int nb, int row_ctas) 
   return (int64_t)g * nb <= cap ? g : 0;
 }
 
-// Enqueues the resident schedule of a batch (g CTAs per solve).
-int enqueue_resident(epfft_ctx* c, Arena& A, Batch& B, int g) {
+// Enqueues the resident schedule of a batch (g CTAs per solve); B.resident
+// tells whether it was: where its scratch cannot be had or the device refuses the
+// cooperative launch, nothing has touched the solves and the two-pass loop,
+// which needs neither, can run them.
+void enqueue_resident(epfft_ctx* c, Arena& A, Batch& B, int g) {
   const size_t part = sizeof(double) * PART_STRIDE * (size_t)B.sh.row_ctas * (size_t)B.nb;
   const size_t bar = 128 * (size_t)B.nb;
   double* part2 = (double*)A.get(part);
-  unsigned* bars = (unsigned*)A.get(bar);
-  if (!part2 || !bars) return EPFFT_ERR_OOM;
-  CK(cudaMemsetAsync(bars, 0, bar, c->stream));
-  if (B.prec == EPFFT_FP64)
-    CK(launch_resident<double>(B.L, B.var, g, B.nb, c->stream, B.d_solves, B.d_ctl, part2, bars, B.tw, B.ktab, B.general));
-  else
-    CK(launch_resident<float>(B.L, B.var, g, B.nb, c->stream, B.d_solves, B.d_ctl, part2, bars, B.tw, B.ktab, B.general));
-  B.resident = true;
-  return EPFFT_OK;
+  unsigned* bars = part2 ? (unsigned*)A.get(bar) : nullptr;
+  if (!bars || cudaMemsetAsync(bars, 0, bar, c->stream) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  const cudaError_t e =
+      B.prec == EPFFT_FP64
+          ? launch_resident<double>(B.L, B.var, g, B.nb, c->stream, B.d_solves, B.d_ctl, part2, bars, B.tw, B.ktab, B.general)
+          : launch_resident<float>(B.L, B.var, g, B.nb, c->stream, B.d_solves, B.d_ctl, part2, bars, B.tw, B.ktab, B.general);
+  if (e != cudaSuccess) cudaGetLastError();
+  B.resident = e == cudaSuccess;
 }
 
 // Runs the device-side loop of a batch to completion (one graph launch).  A
@@ -1324,11 +1329,15 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
     Bp[g] = &Bs[g];
   }
   const char* chk = getenv("EPFFT_SYNC_CHECK");
+  const bool checked = chk && chk[0] == '1';
+  if (!checked && G == 1)
+    if (const int g = resident_ctas(c, Bs[0].L, Bs[0].prec, Bs[0].var, Bs[0].nb, Bs[0].sh.row_ctas))
+      enqueue_resident(c, A, Bs[0], g);
   int rc = EPFFT_OK;
-  if (chk && chk[0] == '1') {
+  if (checked) {
     for (int g = 0; g < G && !rc; g++) rc = run_checked(c, Bs[g]);
-  } else if (const int g = G == 1 ? resident_ctas(c, Bs[0].L, Bs[0].prec, Bs[0].var, Bs[0].nb, Bs[0].sh.row_ctas) : 0) {
-    rc = enqueue_resident(c, A, Bs[0], g);
+  } else if (Bs[0].resident) {
+    // the whole solves are enqueued
   } else if (host_steps > 0) {
     rc = run_host_loop(c, Bs[0], host_steps);
   } else {
@@ -1585,11 +1594,11 @@ int time_resident(epfft_ctx* ctx, epfft_problem p, int n_batch, const double E[4
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
   CK(cudaEventRecord(e0, ctx->stream));
-  rc = enqueue_resident(ctx, A, B, g);
-  if (!rc && (cudaEventRecord(e1, ctx->stream) != cudaSuccess || cudaStreamSynchronize(ctx->stream) != cudaSuccess))
+  enqueue_resident(ctx, A, B, g);
+  if (cudaEventRecord(e1, ctx->stream) != cudaSuccess || cudaStreamSynchronize(ctx->stream) != cudaSuccess)
     rc = EPFFT_ERR_CUDA;
   float t = 0.f;
-  if (!rc && cudaEventElapsedTime(&t, e0, e1) != cudaSuccess) rc = EPFFT_ERR_CUDA;
+  if (!rc && B.resident && cudaEventElapsedTime(&t, e0, e1) != cudaSuccess) rc = EPFFT_ERR_CUDA;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (!rc) *ms = t / (float)n_iter;
