@@ -115,7 +115,6 @@ enum MatConst : int {
   MC_EM_MAT,      // 1 / (9 (K + K0))
   MC_EM_VOID,     // 1 / (9 K0)
   MC_PB_EL,       // (mu - mu0) / (mu + mu0): MC_GSC_EL - 2 mu0 / (2 (mu + mu0))
-  MC_EM_NEAR,     // 2^16 Y / (2 mu): mean strains above it leave the deviator few exact bits
   N_MC
 };
 

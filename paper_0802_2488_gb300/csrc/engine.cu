@@ -415,7 +415,6 @@ void fill_consts(Solve& S) {
   c[MC_EM_MAT] = 1.0 / (9.0 * (K + K0));
   c[MC_EM_VOID] = 1.0 / (9.0 * K0);
   c[MC_PB_EL] = (S.mu - S.mu0) / (S.mu + S.mu0);
-  c[MC_EM_NEAR] = 65536.0 * S.Y / (2.0 * S.mu);
   for (int i = 0; i < N_MC; i++) S.mcf[i] = (float)c[i];
 }
 

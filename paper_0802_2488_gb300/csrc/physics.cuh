@@ -22,9 +22,8 @@ struct Mat {
   T k3;             // 3 K
   // double precision (local_step64): 3 K0, |tau'|^2 / 2 at yield,
   // sqrt(2/3) Y / sqrt(2), mean parts of the strain per trace of tau, elastic
-  // coefficient of the polarization's deviator, bound of the mean strain in
-  // the plastic count, prescribed E33
-  T k03, hlim, ylim_r2, em_mat, em_void, pb_el, em_near, E33;
+  // coefficient of the polarization's deviator, prescribed E33
+  T k03, hlim, ylim_r2, em_mat, em_void, pb_el, E33;
 };
 
 template <typename T>
@@ -60,7 +59,6 @@ __device__ __forceinline__ Mat<T> make_mat(const Solve& S) {
   m.em_mat = c[MC_EM_MAT];
   m.em_void = c[MC_EM_VOID];
   m.pb_el = c[MC_PB_EL];
-  m.em_near = c[MC_EM_NEAR];
   m.E33 = T(0);  // set by the passes that use it
   return m;
 }
@@ -249,9 +247,10 @@ __device__ __forceinline__ bool local_solve_p(const T t[4], bool is_void, const 
 // a record is the number of its flags.  The branch answers it away from the
 // threshold (the strain's deviator grows with |tau'|, and faster beyond yield):
 // within 2^-16 of it in h, for a mean strain whose rounding could reach
-// that far (2^16 times the deviator at yield), and for infinities and NaN,
-// the test itself is evaluated.  (Evaluated at every pixel its dozen FP64
-// instructions would add a fifth to the step's.)
+// that far (2^16 times the deviator at yield, sqrt(2 hlim) / (2 (mu + mu0)),
+// by its exponent), and for infinities and NaN, the test itself is evaluated.
+// (Evaluated at every pixel its dozen FP64 instructions would add a fifth to
+// the step's.)
 __device__ __forceinline__ bool local_step64(const double s[4], double e11, double e22, double e12, bool is_void,
                                              const Mat<double>& m, double e1[4], double s1[4], double p[3]) {
   const double trE = (e11 + e22) + m.E33, trS = (s[0] + s[1]) + s[2];
@@ -279,9 +278,11 @@ __device__ __forceinline__ bool local_step64(const double s[4], double e11, doub
     pb = fma(2.0, gsc, -1.0);  // gsc - 2 mu0 sc
   }
   const double em = t * (is_void ? m.em_void : m.em_mat);
+  // (beyond the exponents' range it wraps to a negative number: always evaluated)
+  const int em_near = (int)((unsigned)((__double2hiint(m.hlim) - 0x3ff00000) >> 1) +
+                            (unsigned)__double2hiint(m.inv_2mumu0) + (16u << 20));
   const unsigned hh = (unsigned)__double2hiint(h), eh = (unsigned)__double2hiint(em) & 0x7fffffffu;
-  const bool near = hh - (unsigned)__double2hiint(m.hlim) + 16u <= 32u || hh >= 0x7ff00000u ||
-                    eh > (unsigned)__double2hiint(m.em_near);
+  const bool near = hh - (unsigned)__double2hiint(m.hlim) + 16u <= 32u || hh >= 0x7ff00000u || (int)eh > em_near;
   const double sm = (is_void ? 0.0 : m.k3) * em, pm = (is_void ? m.p_void : m.p_mat) * em;
   e1[0] = fma(d0, sc, em);
   e1[1] = fma(d1, sc, em);

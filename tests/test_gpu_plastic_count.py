@@ -42,3 +42,19 @@ def test_count_equals_the_flags_of_a_porous_lattice(L):
         for rec, f in zip(recs, fs):
             assert [int(x) for x in rec["n_plastic"]] == [int(p.sum()) for p in f.plastic]
             assert rec["n_plastic"][-1] > 0
+
+
+@pytest.mark.parametrize("big", [1e3, 1e6, 1e12, 1e16])
+def test_count_equals_the_flags_under_a_large_mean_strain(big):
+    """A mean strain far above the yield deviator leaves the stored deviator few
+    exact bits: the branch taken and the flags' test part at any distance."""
+    from paper_0802_2488_gb300 import binding as B
+    rng = np.random.default_rng(3)
+    with B.Context(0) as ctx:
+        for i in range(30):
+            mu, lam, Y = rng.uniform(0.5, 2.0, 3)
+            E = _yield_path(rng, mu, Y) * rng.uniform(0.5, 1.5)
+            E[:, :3] += big * Y
+            prob = B.Problem(L=16, precision="fp64", mu=mu, lambda_=lam, yield_stress=Y, max_iter=20)
+            _, rec, f = B.epfft_solve(ctx, prob, E, fields=True)
+            assert [int(x) for x in rec["n_plastic"]] == [int(p.sum()) for p in f.plastic], i
