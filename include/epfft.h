@@ -276,7 +276,9 @@ int epfft_solve_dg2(epfft_ctx *ctx, const epfft_problem *problem, const epfft_pa
  * n_img*L*L): the final clusters, label = smallest linear index, -1 off
  * the phase.  stats (host, n_img x 6): clusters, pixels of the largest,
  * clusters without a plastic pixel (isolated voids), clusters of the voids
- * alone, plastic pixels, void pixels.  Blocking. */
+ * alone, plastic pixels, void pixels.  Takes 26 bytes of scratch per pixel of
+ * as many images at a time as 512 MB hold, fewer (down to one) where that
+ * cannot be had.  Blocking. */
 int epfft_void_plastic(epfft_ctx *ctx, int32_t L, int32_t n_img, const uint8_t *mask_dev,
                        const uint8_t *plastic_dev, int32_t *labels_dev, int32_t *stats);
 

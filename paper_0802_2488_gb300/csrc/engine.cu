@@ -171,6 +171,15 @@ struct Arena {
     if (p) blocks.push_back({p, bytes});
     return p;
   }
+  // Scratch for as many of `step` units as can be had, halved down to one;
+  // null if not even that.
+  void* get_units(size_t bytes_per_unit, size_t& step) {
+    for (;;) {
+      void* p = get(bytes_per_unit * step);
+      if (p || step <= 1) return p;
+      step = (step + 1) / 2;
+    }
+  }
   ~Arena() {
     cudaStreamSynchronize(c->stream);
     for (auto& b : blocks) dev_free(c, b.first, b.second);
@@ -1178,12 +1187,12 @@ __global__ void __launch_bounds__(256) accepted_strain_kernel(const Solve* S, co
 
 // Enqueues the cluster counts of every increment of a batch (flags of all
 // solves in a row) and their copy into `counts`, followed by the labelling's
-// error flag; up to 256 MB of label scratch at a time.
+// error flag; up to 256 MB of label scratch at a time, less where that cannot be
+// had.
 int count_clusters(epfft_ctx* c, Arena& A, Batch& B, std::vector<int32_t>& counts, int* launches) {
   const size_t LL = (size_t)B.L * B.L;
   size_t step = std::max<size_t>(1, std::min(B.tot_inc, ((size_t)256 << 20) / (sizeof(int32_t) * LL)));
-  int32_t* lab = (int32_t*)A.get(sizeof(int32_t) * LL * step);
-  if (!lab && step > 1) lab = (int32_t*)A.get(sizeof(int32_t) * LL * (step = 1));
+  int32_t* lab = (int32_t*)A.get_units(sizeof(int32_t) * LL, step);
   int32_t* dc = (int32_t*)A.get(sizeof(int32_t) * (B.tot_inc + 1));
   if (!lab || !dc) return EPFFT_ERR_OOM;
   CK(cudaMemsetAsync(dc + B.tot_inc, 0, sizeof(int32_t), c->stream));
@@ -2159,9 +2168,9 @@ int epfft_void_plastic(epfft_ctx* ctx, int32_t L, int32_t n_img, const uint8_t* 
   // images at a time: up to 512 MB of labels and scratch, fewer (down to one)
   // if that cannot be had
   const size_t per = LL * (sizeof(int32_t) + VP_SCRATCH_BYTES);
-  int64_t step = std::max<int64_t>(1, std::min<int64_t>(n_img, (int64_t)(((size_t)512 << 20) / per)));
-  char* buf = (char*)A.get(per * (size_t)step);
-  if (!buf && step > 1) buf = (char*)A.get(per * (size_t)(step = 1));
+  size_t units = std::max<size_t>(1, std::min<size_t>((size_t)n_img, ((size_t)512 << 20) / per));
+  char* buf = (char*)A.get_units(per, units);
+  const int64_t step = (int64_t)units;
   // counts: 4 per image, then clusters and pixels of the voids, the error flag
   const size_t ncnt = 4 * (size_t)n_img + 3;
   int32_t* dcnt = (int32_t*)A.get(ncnt * sizeof(int32_t));

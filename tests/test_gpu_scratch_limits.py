@@ -55,3 +55,31 @@ def test_small_solve_without_the_resident_schedules_scratch(hook, prec, L, tilin
             assert B.epfft_last_stats(ctx)["kernel_launches"] > resident + 10
             assert rc2 == rc and rec2.tobytes() == rec.tobytes()
             assert np.array_equal(f2.eps, f.eps) and np.array_equal(f2.labels, f.labels)
+
+
+def test_cluster_counts_and_void_plastic_take_what_scratch_there_is(hook):
+    """A refused size is halved until it can be had: with 3 images' worth there,
+    8 images are labelled 2 at a time and not one by one."""
+    import torch
+    from paper_0802_2488_gb300 import binding as B
+    from paper_0802_2488_gb300 import inputs
+    L, n = 64, 8
+    g = torch.Generator(device="cuda").manual_seed(4)
+    mask = (torch.rand((L, L), generator=g, device="cuda") < 0.2).to(torch.uint8)
+    plastic = ((torch.rand((n, L, L), generator=g, device="cuda") < 0.4) & (mask == 0)).to(torch.uint8)
+    with B.Context(0) as ctx:
+        ref, lab = B.epfft_void_plastic(ctx, mask, plastic, labels=True)
+        per = 26 * L * L
+        hook.reset(lambda i, s: s > 3 * per)
+        got, lab2 = B.epfft_void_plastic(ctx, mask, plastic, labels=True)
+        assert hook.granted[0] == 2 * per
+        assert np.array_equal(got, ref) and torch.equal(lab, lab2)
+        # a solve without fields counts the clusters of its increments' flags
+        prob = B.Problem(L=L, precision="fp64", void_fraction=0.2, seed=1, max_iter=20)
+        path = inputs.load_path("shear", n, 3.0)
+        _, rec = B.epfft_solve(ctx, prob, path)
+        per = 4 * L * L
+        hook.reset(lambda i, s: s == n * per)
+        _, rec2 = B.epfft_solve(ctx, prob, path)
+        assert n * per in hook.sizes and n // 2 * per in hook.granted
+        assert rec.tobytes() == rec2.tobytes()
