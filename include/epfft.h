@@ -508,7 +508,10 @@ int epfft_fp64_peak(epfft_ctx *ctx, double *tflops, int32_t *n_sm, float *ms);
  * fastest the context's tiling for (L, precision) and for batches of that
  * class: launches that cover at least 2^21 pixels (L^2 x batch) form one
  * class, smaller ones the other, since small launches favour more and
- * smaller CTAs and large ones fewer and larger.  *chosen receives the
+ * smaller CTAs and large ones fewer and larger.  Projections, serving classes
+ * and the refreshes of the defect form take the fastest by its two passes
+ * alone, where whole solves of the size run as one cooperative launch.  *chosen
+ * receives the
  * choice and ms_per_iteration[EPFFT_N_TILINGS] (optional) the timings (0 for
  * a tiling that is not compiled).  Later solves, batches, projections (class
  * of one solve) and serving classes (class of their slot count) of that size

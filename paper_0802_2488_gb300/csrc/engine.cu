@@ -72,6 +72,9 @@ struct epfft_ctx {
   // tuned tiling per (L, precision, batch class): class 1 when a launch
   // covers at least 2^21 pixels (enough CTAs to fill the GPU), else 0
   std::map<std::tuple<int, int, int>, int> variant;
+  // the fastest by its two passes alone, where that is another one (projections,
+  // serving and refreshes never run the resident schedule)
+  std::map<std::tuple<int, int, int>, int> pass_choice;
   // resident schedule: CTAs the GPU holds at once per (L, precision, tiling)
   std::map<std::tuple<int, int, int>, int> res_cap;
   epfft_stats last{};
@@ -356,11 +359,20 @@ int batch_class(int L, int nb) { return (int64_t)L * L * nb >= ((int64_t)1 << 21
 
 int variant_for(epfft_ctx* c, int L, int prec, int nb);
 
-// The tuned tiling where the two passes run (projections, serving, the
-// fixed-step loops): the on-chip schedule maps to tiling 0.
-int pass_variant(epfft_ctx* c, int L, int prec, int nb) {
+// The tuned tiling of whole solves and fixed-step loops without the on-chip
+// schedule, which maps to tiling 0.  (Calls of several groups and batches
+// past the resident schedule's limit take it too, so that a problem's numbers
+// do not depend on the others of its call.)
+int stream_variant(epfft_ctx* c, int L, int prec, int nb) {
   const int v = variant_for(c, L, prec, nb);
   return v == ONCHIP_VARIANT ? 0 : v;
+}
+
+// The tuned tiling where the passes run by themselves (projections, serving,
+// the defect form's refresh).
+int pass_variant(epfft_ctx* c, int L, int prec, int nb) {
+  auto it = c->pass_choice.find(std::make_tuple(L, prec, batch_class(L, nb)));
+  return it == c->pass_choice.end() ? stream_variant(c, L, prec, nb) : it->second;
 }
 
 int variant_for(epfft_ctx* c, int L, int prec, int nb) {
@@ -658,7 +670,7 @@ int setup_batch(epfft_ctx* c, Arena& A, Batch& B, int n, const epfft_problem* pr
   B.prec = probs[0].precision;
   B.nb = n;
   for (int i = 0; i < n; i++) B.general |= probs[i].green != EPFFT_GREEN_EQ3;
-  if (B.var < 0) B.var = onchip ? variant_for(c, B.L, B.prec, n) : pass_variant(c, B.L, B.prec, n);
+  if (B.var < 0) B.var = onchip ? variant_for(c, B.L, B.prec, n) : stream_variant(c, B.L, B.prec, n);
   int rc = shape(B.L, B.prec, B.var, &B.sh);
   if (rc) return rc;
   rc = get_tables(c, B.L, table_prec(B.prec), &B.tw, &B.ktab);
@@ -666,7 +678,7 @@ int setup_batch(epfft_ctx* c, Arena& A, Batch& B, int n, const epfft_problem* pr
   if (!rc && B.prec == EPFFT_FP32_DEFECT) {
     // the refresh: FP64 tables, FP64 column pass and FP64 row halves of the
     // FP64 tiling tuned for this batch class
-    B.var64 = variant_for(c, B.L, EPFFT_FP64, n);
+    B.var64 = pass_variant(c, B.L, EPFFT_FP64, n);
     rc = get_tables(c, B.L, EPFFT_FP64, &B.tw64, &B.ktab64);
     if (!rc) rc = ensure_prepared(c, B.L, EPFFT_FP64, B.var64);
     if (!rc) rc = ensure_prepared(c, B.L, EPFFT_FP32_DEFECT, B.var64);
@@ -1579,16 +1591,21 @@ int time_passes_impl(epfft_ctx* ctx, epfft_problem p, int n_batch, const double 
   return EPFFT_OK;
 }
 
-// Time per iteration (ms) of a solve of n_batch copies of p on the resident
-// schedule with tiling var: one launch of n_iter iterations.  *ms = 0 where
-// that batch runs the two-pass loop.
-int time_resident(epfft_ctx* ctx, epfft_problem p, int n_batch, const double E[4], int n_iter, int var, float* ms) {
+// CTAs per solve of the resident schedule for n_batch copies of p with tiling
+// var, 0 where they run the two-pass loop.
+int resident_tiling(epfft_ctx* ctx, const epfft_problem& p, int n_batch, int var) {
+  PassShape sh;
+  if (var == ONCHIP_VARIANT || shape(p.L, p.precision, var, &sh) != EPFFT_OK) return 0;
+  return resident_ctas(ctx, p.L, p.precision, var, n_batch, sh.row_ctas);
+}
+
+// Time per iteration (ms) of a whole solve of n_batch copies of p with tiling
+// var, n_iter iterations by the schedule such a solve takes: the resident one,
+// or the graph of the two-pass loop.
+int time_solve(epfft_ctx* ctx, epfft_problem p, int n_batch, const double E[4], int n_iter, int var, float* ms) {
   *ms = 0.f;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return EPFFT_ERR_CUDA;
-  PassShape sh;
-  if (var == ONCHIP_VARIANT || shape(p.L, p.precision, var, &sh) != EPFFT_OK) return EPFFT_OK;
-  const int g = resident_ctas(ctx, p.L, p.precision, var, n_batch, sh.row_ctas);
-  if (!g) return EPFFT_OK;
+  const int g = resident_tiling(ctx, p, n_batch, var);
   p.tol_eq = p.tol_macro = 0.0;
   p.max_iter = n_iter;
   std::vector<epfft_problem> ps(n_batch, p);
@@ -1597,19 +1614,30 @@ int time_resident(epfft_ctx* ctx, epfft_problem p, int n_batch, const double E[4
   Batch B;
   B.var = var;
   int rc = setup_batch(ctx, A, B, n_batch, ps.data(), paths.data(), nullptr);
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+  if (!rc && !g) rc = build_loop_graph(ctx, B, &graph, &exec);
   if (rc) return rc;
-  cudaEvent_t e0, e1;
-  CK(cudaEventCreate(&e0));
-  CK(cudaEventCreate(&e1));
-  CK(cudaEventRecord(e0, ctx->stream));
-  enqueue_resident(ctx, A, B, g);
-  if (cudaEventRecord(e1, ctx->stream) != cudaSuccess || cudaStreamSynchronize(ctx->stream) != cudaSuccess)
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess ||
+      cudaEventRecord(e0, ctx->stream) != cudaSuccess)
     rc = EPFFT_ERR_CUDA;
+  if (!rc && g) {
+    enqueue_resident(ctx, A, B, g);
+    if (!B.resident) rc = EPFFT_ERR_CUDA;
+  } else if (!rc && cudaGraphLaunch(exec, ctx->stream) != cudaSuccess) {
+    rc = EPFFT_ERR_CUDA;
+  }
+  if (!rc && cudaEventRecord(e1, ctx->stream) != cudaSuccess) rc = EPFFT_ERR_CUDA;
+  if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) rc = EPFFT_ERR_CUDA;
   float t = 0.f;
-  if (!rc && B.resident && cudaEventElapsedTime(&t, e0, e1) != cudaSuccess) rc = EPFFT_ERR_CUDA;
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  if (!rc) *ms = t / (float)n_iter;
+  if (!rc && cudaEventElapsedTime(&t, e0, e1) != cudaSuccess) rc = EPFFT_ERR_CUDA;
+  if (e0) cudaEventDestroy(e0);
+  if (e1) cudaEventDestroy(e1);
+  if (exec) cudaGraphExecDestroy(exec);
+  if (graph) cudaGraphDestroy(graph);
+  if (rc) cudaGetLastError();
+  else *ms = t / (float)n_iter;
   return rc;
 }
 
@@ -1746,7 +1774,7 @@ int get_class(epfft_ctx* c, Server& S, int L, int prec, int general, ServeClass*
   if (!rc) rc = ensure_prepared(c, L, prec, B.var);
   if (!rc && prec == EPFFT_FP32_DEFECT) {
     // the refresh between serving steps (FP64 tables, column pass, row halves)
-    B.var64 = variant_for(c, L, EPFFT_FP64, S.cap);
+    B.var64 = pass_variant(c, L, EPFFT_FP64, S.cap);
     rc = get_tables(c, L, EPFFT_FP64, &B.tw64, &B.ktab64);
     if (!rc) rc = ensure_prepared(c, L, EPFFT_FP64, B.var64);
     if (!rc) rc = ensure_prepared(c, L, EPFFT_FP32_DEFECT, B.var64);
@@ -2857,30 +2885,47 @@ int epfft_autotune(epfft_ctx* ctx, int32_t L, int32_t precision, int32_t n_batch
   const double E[4] = {0.0, 0.0, 0.0, 1.5 / (2.0 * std::sqrt(3.0))};
   const int64_t px = (int64_t)L * L * n_batch;
   const int n_iter = px >= ((int64_t)1 << 24) ? 10 : 30;
-  int best = -1;
-  float tbest = 0.f;
+  // where some tiling runs the resident schedule for this batch, every one is
+  // timed as whole solves (the on-chip schedule always is); else by its two
+  // passes
+  bool whole = false;
+  for (int v = 0; v < N_VARIANTS; v++) whole |= resident_tiling(ctx, p, n_batch, v) > 0;
+  int best = -1, pbest = -1;
+  float tbest = 0.f, tpbest = 0.f;
   for (int v = 0; v < N_VARIANTS; v++) {
     if (ms_per_iteration) ms_per_iteration[v] = 0.f;
     PassShape sh;
     if (shape(L, precision, v, &sh) != EPFFT_OK) continue;  // not compiled for this size
     float c = 0.f, r = 0.f;
     // warm-up, then the timed launches
-    // a batch that runs on the resident schedule is timed on it
-    int rc = time_resident(ctx, p, n_batch, E, 3, v, &r);
-    if (!rc && r > 0.f) {
-      rc = time_resident(ctx, p, n_batch, E, n_iter, v, &r);
-    } else if (!rc) {
-      rc = time_passes_impl(ctx, p, n_batch, E, 3, v, &c, &r);
-      if (!rc) rc = time_passes_impl(ctx, p, n_batch, E, n_iter, v, &c, &r);
-    }
+    int rc = time_passes_impl(ctx, p, n_batch, E, 3, v, &c, &r);
+    // (few launches where they only choose between the passes' tilings)
+    const int n = whole && v != ONCHIP_VARIANT ? std::min(n_iter, 8) : n_iter;
+    if (!rc) rc = time_passes_impl(ctx, p, n_batch, E, n, v, &c, &r);
     if (rc) return rc;
-    if (ms_per_iteration) ms_per_iteration[v] = c + r;
-    if (best < 0 || c + r < tbest) {
-      tbest = c + r;
+    float t = c + r;
+    if (v != ONCHIP_VARIANT) {
+      if (pbest < 0 || t < tpbest) {
+        tpbest = t;
+        pbest = v;
+      }
+      if (whole) {
+        rc = time_solve(ctx, p, n_batch, E, 3, v, &t);
+        if (!rc) rc = time_solve(ctx, p, n_batch, E, n_iter, v, &t);
+        if (rc) return rc;
+      }
+    }
+    if (ms_per_iteration) ms_per_iteration[v] = t;
+    if (best < 0 || t < tbest) {
+      tbest = t;
       best = v;
     }
   }
-  ctx->variant[std::make_tuple((int)L, (int)precision, batch_class(L, n_batch))] = best;
+  const auto key = std::make_tuple((int)L, (int)precision, batch_class(L, n_batch));
+  ctx->variant[key] = best;
+  // (with the on-chip schedule the passes take tiling 0, as documented)
+  if (best != ONCHIP_VARIANT) ctx->pass_choice[key] = pbest;
+  else ctx->pass_choice.erase(key);
   if (chosen) *chosen = best;
   return EPFFT_OK;
 }
@@ -2897,7 +2942,11 @@ int epfft_set_tiling(epfft_ctx* ctx, int32_t L, int32_t precision, int32_t varia
     return EPFFT_ERR_ARG;
   if (!supported(L, precision)) return EPFFT_ERR_UNSUPPORTED;
   if (!epfft_supported_tiling(L, precision, variant)) return EPFFT_ERR_UNSUPPORTED;
-  for (int k = 0; k < 2; k++) ctx->variant[std::make_tuple((int)L, (int)precision, k)] = variant;
+  for (int k = 0; k < 2; k++) {
+    const auto key = std::make_tuple((int)L, (int)precision, k);
+    ctx->variant[key] = variant;
+    ctx->pass_choice.erase(key);
+  }
   return EPFFT_OK;
 }
 
