@@ -503,17 +503,20 @@ def roofline(precision, L, nb, col_ms, row_ms, peak, peak_source, tiling=None):
     Defect form (HBM): row pass 113 (spectrum 24, the stress difference of
     iterate n read 16, the new strain and stress differences written 32, the
     reference data read 40, mask 1), column pass 24.
-    FP64 (FP64 ALU): flops per pixel, row pass 15 log2 L + 60 (row
-    transforms, local step), column pass 15 log2 L + 25 (column transforms,
-    Green operator); the transforms' flops are done in 64-bit integers, so the
-    fraction of the FP64 peak can exceed 1."""
+    FP64: flops per pixel, row pass 15 log2 L + 60 (row transforms, local
+    step), column pass 15 log2 L + 25 (column transforms, Green operator).  The
+    transforms' are done in 64-bit integers, so `frac`, the fraction of the
+    FP64 peak, counts the 60 and the 25 alone (`fp64_alu_work_per_launch`);
+    `achieved` is the rate of all."""
     n = L * L * nb
     lg = int(np.log2(L))
     if precision in ("fp32", "fp32_defect"):
         work = {"row": (73 if precision == "fp32" else 113) * n, "col": 24 * n}
         unit, scale, bound = "GB/s", 1e9, "hbm"
+        piped = work
     else:
         work = {"row": (15 * lg + 60) * n, "col": (15 * lg + 25) * n}
+        piped = {"row": 60 * n, "col": 25 * n}
         unit, scale, bound = "TFLOP/s", 1e12, "alu"
     ms = {"row": row_ms, "col": col_ms}
     names = pass_kernels(precision, L, tiling)
@@ -521,8 +524,11 @@ def roofline(precision, L, nb, col_ms, row_ms, peak, peak_source, tiling=None):
     for k in ("row", "col"):
         a = work[k] / (ms[k] * 1e-3) / scale
         tr = traffic_of(precision, L, nb, tiling, k)
-        passes[k] = {"kernel": names[k], "ms": ms[k], "achieved": a, "frac": a / peak,
+        passes[k] = {"kernel": names[k], "ms": ms[k], "achieved": a,
+                     "frac": piped[k] / (ms[k] * 1e-3) / scale / peak,
                      "work_per_launch": work[k], "traffic": tr[0] if tr else None}
+        if bound == "alu":
+            passes[k]["fp64_alu_work_per_launch"] = piped[k]
     dom = "row" if row_ms >= col_ms else "col"
     d = passes[dom]
     tr = traffic_of(precision, L, nb, tiling, dom)
@@ -538,7 +544,9 @@ def roofline(precision, L, nb, col_ms, row_ms, peak, peak_source, tiling=None):
             "peak_source": peak_source, "passes": passes,
             "timing": "epfft_time_passes: CUDA events around each launch on the context stream, mean of the "
                       "timed launches, the same launch shape as the solve" +
-                      ("; the transforms' flops of the count are done in 64-bit integers" if bound == "alu" else "")}
+                      ("; frac is the share of the FP64 peak that the flops on the FP64 pipe take (local step, Green "
+                       "operator), achieved counts the transforms, done in 64-bit integers, too"
+                       if bound == "alu" else "")}
 
 
 def solve_line(B, ctx, stream, flush, torch, name, precision, cap, steps, warmup, e2e_steps, local, ws,
