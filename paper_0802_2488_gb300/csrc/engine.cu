@@ -1189,9 +1189,13 @@ int run_checked(epfft_ctx* c, Batch& B) {
 }
 
 // Copies the accepted strain of a finished solve to `out` (words of 16 bytes).
-__global__ void __launch_bounds__(256) accepted_strain_kernel(const Solve* S, const BatchCtl* bc, int4* __restrict__ out,
-                                                              int64_t words) {
+// Left as it is where the call will fail: a self-check fired (checks: the
+// gathered records) or the loop's bound stopped it.
+__global__ void __launch_bounds__(256) accepted_strain_kernel(const Solve* S, const BatchCtl* bc, const CheckRec* checks,
+                                                              int4* __restrict__ out, int64_t words) {
   if (S->phase != PH_DONE || bc->timed_out) return;
+  for (int i = 0; i < N_CHECK_UNITS; i++)
+    if (checks[i].code) return;
   const int4* in = reinterpret_cast<const int4*>(S->eps[S->cur]);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < words; i += (int64_t)gridDim.x * blockDim.x)
     out[i] = in[i];
@@ -1386,11 +1390,12 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
     if (ocs != c->stream && cudaStreamSynchronize(ocs) != cudaSuccess && !rc) rc = EPFFT_ERR_CUDA;
   }
   if (rc) return rc;
-  // behind the loop on the same stream: the accepted strain of a solve whose
-  // caller wants it in place, and, when no fields are asked for, the cluster
-  // counts; then one read-back of the solve states, the control blocks, the
-  // records, the counts and the self-check records
+  // behind the loop on the same stream: the self-check records, the accepted
+  // strain of a solve whose caller wants it in place, and, when no fields are
+  // asked for, the cluster counts; then one read-back of the solve states, the
+  // control blocks, the records and the counts
   int launches = 1;  // the gathering of the self-check records
+  CK(enqueue_check_reads(c, c->stream));
   // (a caller's buffer off the 16-byte boundary is copied after the read-back)
   auto aligned = [&](int i) { return ((uintptr_t)eps_out[i] & 15) == 0; };
   if (eps_out)
@@ -1399,7 +1404,7 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
         Batch& B = Bs[where[i]];
         const int64_t words = (int64_t)B.L * B.L * (int64_t)real_size(B.prec) / 4;
         accepted_strain_kernel<<<(unsigned)std::min<int64_t>((words + 255) / 256, 152 * 16), 256, 0, c->stream>>>(
-            B.d_solves + slot[i], B.d_ctl, (int4*)eps_out[i], words);
+            B.d_solves + slot[i], B.d_ctl, c->d_checks, (int4*)eps_out[i], words);
         if (cudaGetLastError() != cudaSuccess) return EPFFT_ERR_CUDA;
         launches++;
       }
@@ -1417,7 +1422,6 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
     CK(A.read(&bc[g], Bs[g].d_ctl, sizeof(BatchCtl)));
     CK(A.read(rec[g].data(), Bs[g].d_rec, sizeof(Record) * Bs[g].tot_inc));
   }
-  CK(enqueue_check_reads(c, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   A.land();
   rc = check_result(c);
