@@ -26,12 +26,14 @@
 // every operation).  A NaN or infinity in a sequence makes every output of it
 // NaN.
 //
-// Measured (8 x L = 512, CUDA events): column pass 581 -> 330 us, row pass
-// 787 -> 631 us, 416 with the twists in fixed point too and the pixel step of
-// local_step64, and 205 and 330 us with the CTA shapes this left room for
+// Measured (8 x L = 512, CUDA events): FP64 butterflies 581 us (column pass) and
+// 787 us (row pass); 207 and 332 us with the transforms and the twists in fixed
+// point, the pixel step of local_step64 and the CTA shapes this left room for
 // (Cfg in passes.cuh); what is left on the FP64 pipe is the Green operator and
-// the pixel step.  L = 4096: 5.69 -> 2.74 ms and 7.83 -> 4.15 ms.
-// Against long double: projection at L = 64, 256 1.8e-16, 1.9e-16 relative
+// the pixel step.  L = 4096: 5.69 -> 2.88 ms and 7.83 -> 4.32 ms.  (One block
+// exponent for all sequences of a call instead of one each: 205 and 330 us, 2.86
+// and 4.25 ms.)
+// Against long double: projection at L = 64, 256 1.8e-16, 1.8e-16 relative
 // (FP64 butterflies 3.2e-16, 3.6e-16), 20 iterations at L = 256 7.0e-16
 // (1.25e-15).
 #pragma once

@@ -63,9 +63,9 @@ struct Cfg {
   static constexpr int RR0 = L <= 64 ? 2 : (L <= 512 || L == 4096 ? 4 : 2);
   static constexpr int RR0_DEF = L <= 64 ? 2 : (L == 2048 ? 8 : 4);
   // FP64 tiling 0: one row of 128 threads at L = 512, four CTAs per SM at 128
-  // registers (8 x L = 512: 324 us; two rows, two CTAs at 191 registers 424;
-  // 2 x 256 threads 358, 4 x 256 351), two rows of 256 at L = 1024 (232 us;
-  // 285 at one CTA per SM), one of 256 at 2048 (940 us; two rows 1070).
+  // registers (8 x L = 512: 332 us; two rows, two CTAs at 191 registers 424;
+  // 2 x 256 threads 358, 4 x 256 351), two rows of 256 at L = 1024 (244 us;
+  // 285 at one CTA per SM), one of 256 at 2048 (970 us; two rows 1070).
   static constexpr int RR64 = L == 512 || L == 2048 ? 1 : 2;
   static constexpr int RR = V == 0 ? (F64 ? RR64 : (DEF ? RR0_DEF : RR0))
                                    : (F64 ? (L <= 256 || L == 4096 ? 1 : 2) : (L <= 256 ? 1 : 2));
@@ -87,16 +87,21 @@ struct Cfg {
                                                : (L <= 128 ? L
                                                            : (L == 256 ? 128
                                                                        : (L == 512 || (L == 1024 && !DEF) ? 256 : 512))));
-  static constexpr int MINB_ROW = F64 ? (V == 0 && L >= 256 && L <= 2048 ? 512 / NT_ROW0 : 1) : (V == 1 ? 2 : (L >= 128 && L <= 2048 ? 1024 / NT_ROW0 : 1));
+  // FP64 rows: 512 threads per SM (128 registers) in tiling 0 from L = 64 to 2048
+  // and in tiling 1 at L = 256, whose rows are a few registers above it otherwise
+  // (L = 128, 37 lattices: 12.4 ms a solve at 132 registers, 11.6 at 128)
+  static constexpr bool F64_128 = V == 0 ? L >= 64 && L <= 2048 : L == 256;
+  static constexpr int MINB_ROW = F64 ? (F64_128 ? 512 / NT_ROW0 : 1)
+                                      : (V == 1 ? 2 : (L >= 128 && L <= 2048 ? 1024 / NT_ROW0 : 1));
   static constexpr int NT_ROW = NT_ROW0 < 32 ? 32 : NT_ROW0;
   static constexpr int NT_COL0 = ((3 * W * L / RM_COL + 31) / 32) * 32;
   // 256 threads at most for FP64 columns: at 512 the 128 registers of a
   // thread spill at L = 4096 (3.75 ms against 2.74), and one column on 256
   // threads three times per SM (80 registers) beats two on 512 at L = 512
-  // (8 x L = 512: 205 us against 330)
+  // (8 x L = 512: 207 us against 330)
   static constexpr int NTMAX_COL = F64 ? 256 : NTMAX;
   static constexpr int NT_COL = NT_COL0 < 32 ? 32 : (NT_COL0 > NTMAX_COL ? NTMAX_COL : NT_COL0);
-  // FP64: 768 threads per SM up to L = 512, 512 at L = 1024 (244 -> 170 us)
+  // FP64: 768 threads per SM up to L = 512, 512 at L = 1024 (244 -> 172 us)
   static constexpr int MINB_COL = F64 ? (L <= 512 ? 768 / NT_COL : (L == 1024 ? 2 : 1))
                                       : V == 1 ? 2 : (L == 512 ? 768 / NT_COL : (L == 1024 || L == 2048 ? 3 : 1));
   // sequences transformed per call: the largest divisor of the sequence
@@ -332,12 +337,14 @@ struct RowIO {
     reinterpret_cast<C2<i64>*>(s)[0] = mk(rshift<2>(a + b), rshift<2>(a - b));
   }
   static __device__ __forceinline__ void c2r_twist64(C2<T>* sp, const C2<T>* __restrict__ oct, int* em) {
-    constexpr int HK = M / 2;
+    constexpr int HK = M / 2, DS = NT >= HK ? NT / HK : 1, NQ = (NSEQ + DS - 1) / DS;
     unsigned* wm = seq_scratch<NT>().wm;
     const int tid = threadIdx.x;
-    if constexpr (NT >= HK) {
-      // a thread's pairs stay in registers while the exponents are found
-      constexpr int DS = NT / HK, NQ = (NSEQ + DS - 1) / DS;
+    // Up to L = 256 a thread's pairs stay in registers while the exponents are
+    // found (16 x L = 256: 186 us, 188 by the scan); above, where they would take
+    // 24 registers and more, the tile is scanned first (8 x L = 512: 332 us, 340
+    // in registers; L = 1024: 244, 261).
+    if constexpr (NT >= HK && HK <= 64) {
       static_assert(HK <= 32 || NSEQ * (HK / 32) <= (int)(sizeof(SeqScratch::wm) / sizeof(unsigned)), "slots");
       const int k = 1 + tid % HK, ik = pad32(k), ikk = pad32(M - k);
       const Tw64 wk = twist_tw64<L>(oct, k);
@@ -380,7 +387,7 @@ struct RowIO {
         }
       }
     } else {
-      // the exponents first, by a slot per sequence and warp
+      // by a slot per sequence and warp
       constexpr int SPS = NT / 32;
       static_assert(M % NT == 0 && NSEQ * SPS <= (int)(sizeof(SeqScratch::wm) / sizeof(unsigned)), "slots");
 #pragma unroll
@@ -779,8 +786,9 @@ __device__ __forceinline__ void finalize_solve(Solve& S, int phase, const double
     const float ss = s0 * s0 + s1 * s1 + 2.0f * s3 * s3, r = rough_float(div2);
     auto fin = [](double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; };
     // finite, normal numbers only: the FP64 path decides the rest
-    far = fin(S.sig_prev[0]) && fin(S.sig_prev[1]) && fin(S.sig_prev[3]) && ss > 1e-30f && ss < 1e30f && den > 1e-30f && den < 1e30f && r < 1e30f && d < 1e30f &&
-          d > (1.001f * tol * tol + 1e-34f) * den && d > 1e-30f;
+    far = fin(S.sig_prev[0]) && fin(S.sig_prev[1]) && fin(S.sig_prev[3]) && ss > 1e-30f && ss < 1e30f &&
+          den > 1e-30f && den < 1e30f && r < 1e30f && d > 1e-30f && d < 1e30f &&
+          d > (1.001f * tol * tol + 1e-34f) * den;
   }
   if (n >= 1 && !far) {
     const double* E = S.path + 4 * S.inc;

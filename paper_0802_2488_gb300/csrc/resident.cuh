@@ -23,7 +23,7 @@
 // passes the barrier after its sums before any CTA writes that buffer again.
 // Measured, one lattice, us an iteration against the two-pass loop: FP32 L = 16
 // 9.0 / 17.8, 64 9.8 / 20.3, 128 10.7 / 23.3, 256 16.6 / 25.9, 512 25.5 / 31.3;
-// FP64 L = 16 21.6 / 31.9, 64 22.3 / 29.3, 128 25.7 / 33.3 (bound by chains of FP64
+// FP64 L = 16 21.2 / 31.9, 64 22.2 / 29.3, 128 25.8 / 33.3 (bound by chains of FP64
 // instructions, 64 clocks each).
 //
 // Every CTA of a launch is resident at once (cooperative launch), and every
