@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(CCL_NT) ccl_roots(int32_t* lab, const uint8_t*
 
 static int grid_for(int64_t n) {
   int64_t g = (n + 255) / 256;
-  if (g > 152 * 32) g = 152 * 32;
+  if (g > GRID_SMS * 32) g = GRID_SMS * 32;
   if (g < 1) g = 1;
   return (int)g;
 }
@@ -238,7 +238,7 @@ static cudaError_t tile_launch(const uint8_t* flags, const uint8_t* mask, int32_
 // CTAs over one image's pixels and over the images
 static dim3 image_grid(int64_t px, int64_t n_img) {
   const int64_t y = n_img < 32768 ? n_img : 32768;
-  int64_t x = (px + 4 * CCL_NT - 1) / (4 * CCL_NT), most = (152 * 16 + y - 1) / y;
+  int64_t x = (px + 4 * CCL_NT - 1) / (4 * CCL_NT), most = (GRID_SMS * 16 + y - 1) / y;
   if (x > most) x = most;
   return dim3((unsigned)(x < 1 ? 1 : x), (unsigned)y);
 }

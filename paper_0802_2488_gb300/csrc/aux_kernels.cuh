@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 namespace epfft {
+constexpr int GRID_SMS = 152;  // SMs of a GB300: caps of grid sizes, nothing depends on it
 #ifdef __CUDACC__
 // Pixel i is a void iff (SplitMix64 output i of `seed`) >> 11 < thr, where the
 // i-th output of SplitMix64 is the 64-bit finaliser of seed + (i+1) gamma,

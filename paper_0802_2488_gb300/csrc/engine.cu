@@ -766,7 +766,7 @@ int setup_batch(epfft_ctx* c, Arena& A, Batch& B, int n, const epfft_problem* pr
   B.d_shadow = dc ? (Solve*)(up + o_shadow) : nullptr;
   B.d_ctl = (BatchCtl*)(up + o_ctl);
   if (init) {
-    const int64_t q = ((int64_t)LL / 4 + 255) / 256, most = std::max<int64_t>(1, 152 * 16 / n);
+    const int64_t q = ((int64_t)LL / 4 + 255) / 256, most = std::max<int64_t>(1, GRID_SMS * 16 / n);
     // grid.y holds at most 65535 solves
     for (int i0 = 0; i0 < n; i0 += 65535) {
       batch_init_kernel<<<dim3((unsigned)std::min(q, most), (unsigned)std::min(n - i0, 65535)), 256, 0, c->stream>>>(
@@ -1403,7 +1403,7 @@ int solve_impl(epfft_ctx* c, int32_t n, const epfft_problem* probs, const epfft_
       if (eps_out[i] && aligned(i)) {
         Batch& B = Bs[where[i]];
         const int64_t words = (int64_t)B.L * B.L * (int64_t)real_size(B.prec) / 4;
-        accepted_strain_kernel<<<(unsigned)std::min<int64_t>((words + 255) / 256, 152 * 16), 256, 0, c->stream>>>(
+        accepted_strain_kernel<<<(unsigned)std::min<int64_t>((words + 255) / 256, GRID_SMS * 16), 256, 0, c->stream>>>(
             B.d_solves + slot[i], B.d_ctl, c->d_checks, (int4*)eps_out[i], words);
         if (cudaGetLastError() != cudaSuccess) return EPFFT_ERR_CUDA;
         launches++;

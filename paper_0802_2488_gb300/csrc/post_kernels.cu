@@ -10,7 +10,7 @@ namespace {
 
 int grid_of(int64_t n) {
   const int64_t g = (n + 255) / 256;
-  return (int)(g < 152 * 16 ? (g < 1 ? 1 : g) : 152 * 16);
+  return (int)(g < GRID_SMS * 16 ? (g < 1 ? 1 : g) : GRID_SMS * 16);
 }
 
 __device__ __forceinline__ int64_t mirror_index(int64_t i, int L, int axes) {
@@ -238,7 +238,7 @@ cudaError_t launch_vp_attach(const uint8_t* mask, const int32_t* lab, int32_t* o
   const int g = grid_of(n * n_img);
   const unsigned gy = (unsigned)(n_img < 32768 ? n_img : 32768);
   // up to 16 pixels a thread in the kernels that sum per image
-  int64_t gx = (n + 4095) / 4096, most = (152 * 8 + gy - 1) / gy;
+  int64_t gx = (n + 4095) / 4096, most = (GRID_SMS * 8 + gy - 1) / gy;
   if (gx < most) gx = (n + 255) / 256 < most ? (n + 255) / 256 : most;
   const dim3 per((unsigned)gx, gy);
   vp_nearest_kernel<<<g, 256, 0, s>>>(mask, lab, vp, n_voids_dev, L, n_img);
